@@ -260,8 +260,9 @@ int wilson_eo_apply_batch_rhs(int n, const wilson_eo_t *hs, void *const *outs,
 
 /* Autotune M_eo on this handle with nrhs right-hand sides: every candidate is
  * timed with CUDA events on `stream` and the fastest is kept -- the two-launch
- * algorithm with threads 64/128/192/256 per CTA and 1, 2 or 4 right-hand sides
- * per thread or 2 on neighbouring lanes (FP32 / 16-bit handles, nrhs >= 2), and
+ * algorithm with its default kernel, with threads 64/128/192/256 per CTA and 2 or
+ * 4 right-hand sides per thread or 2 on neighbouring lanes (FP32 / 16-bit handles,
+ * nrhs >= 2), and
  * for FP32 / 16-bit handles the fused algorithm with a lookahead of 4 or 8
  * t-slices and 128 / 256 threads, and for FP32 18-real handles with nrhs = 1
  * the TMA-staged hop (wilson_eo_get_launch, wilson_eo_get_algorithm,
@@ -384,9 +385,14 @@ int wilson_eo_hop_split(wilson_eo_t h, int ranks, int out_parity, int dag, void 
                         const void *in, void *stream);
 
 /* Launch configuration of the hopping kernels for the handle's precision:
- * threads per block (32..256, a multiple of 32) and right-hand sides per
- * thread (1, 2 or 4; values other than 1 apply to FP32 and 16-bit handles, where the
- * links loaded for a site are shared by that many right-hand sides).
+ * right-hand sides per thread (1, 2 or 4; values other than 1 apply to FP32 and
+ * 16-bit handles, where the links loaded for a site are shared by that many
+ * right-hand sides), and threads per block (32..256, a multiple of 32) of the
+ * kernels that compute a whole site in one thread. With 1 (default) and no other
+ * kernel named, the library chooses by size between a kernel that spreads a
+ * site's directions over four warps, whose CTAs have 128 threads, the
+ * one-site-per-thread kernel, and for several right-hand sides the tiles of
+ * wilson_eo_set_tile_links; the results do not depend on the choice.
  * order 1 (default): the second hop of M_eo walks the sites from the top down,
  * so it first reads the part of the odd intermediate the first hop wrote last,
  * while that part is still in L2; order 0: both hops walk upward.
@@ -423,7 +429,8 @@ int wilson_eo_set_site_blocks(wilson_eo_t h, int blocked);
  * nrhs >= 2 groups), until all nrhs are done; spinors are read from global
  * memory. groups 2, 4 or 8 turns it on for the handle's FP32 or 16-bit hops
  * whenever nrhs >= 2 (and sets one right-hand side per thread for the other
- * kernels); 0 (default) turns it off. WEO_ERR_ARG for other values,
+ * kernels); with 0 (default) the library uses groups of 4 where they are the
+ * faster kernel (see wilson_eo_set_launch). WEO_ERR_ARG for other values,
  * WEO_ERR_UNSUPPORTED on an FP64 handle. wilson_eo_tune times these
  * configurations too. */
 int wilson_eo_set_tile_links(wilson_eo_t h, int groups, int rhs_per_thread);

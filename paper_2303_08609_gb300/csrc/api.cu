@@ -20,6 +20,9 @@ HopParams geom_params(const wilson_eo_s *h)
     p.lz = h->dims[2];
     p.lt = h->dims[3];
     p.vh = (int)h->vh;
+    p.dx = FastDiv(p.lxh);
+    p.dy = FastDiv(p.ly);
+    p.dz = FastDiv(p.lz);
     return p;
 }
 

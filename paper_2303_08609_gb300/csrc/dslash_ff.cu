@@ -88,13 +88,8 @@ template <bool Dag, bool Axpy>
 __device__ __forceinline__ void hop_site_ff(const HopParams &p, const int i, const int rhs)
 {
     constexpr int S0 = Dag ? -1 : 1;
-    int rem = i;
-    const int xh = rem % p.lxh;
-    rem /= p.lxh;
-    const int y = rem % p.ly;
-    rem /= p.ly;
-    const int z = rem % p.lz;
-    const int t = rem / p.lz;
+    int xh, y, z;
+    const int t = p.dz.div(p.dy.div(p.dx.div(i, xh), y), z);
     const int par = (y + z + t + p.out_parity) & 1;
     const int op = p.out_parity, in_par = op ^ 1;
     const int sy = p.lxh, sz = p.lxh * p.ly, st = p.lxh * p.ly * p.lz;

@@ -33,7 +33,7 @@ namespace weo {
 // Intermediate loaders that bypass L1 (same layouts as SpF32 and Sp16).
 struct SpF32L2 : SpF32 {
     template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    __device__ static __forceinline__ NoScale load(const void *base, long long vh, long long i,
                                                 cx<R> v[12])
     {
         const float2 *p = static_cast<const float2 *>(base);
@@ -42,13 +42,14 @@ struct SpF32L2 : SpF32 {
             const float2 d = __ldcg(p + k * vh + i);
             v[k] = {R(d.x), R(d.y)};
         }
+        return NoScale();
     }
 };
 
 template <class Tr>
 struct Sp16L2 : Sp16<Tr> {
     template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    __device__ static __forceinline__ float load(const void *base, long long vh, long long i,
                                                 cx<R> v[12])
     {
         const uint4 *p = static_cast<const uint4 *>(base);
@@ -57,11 +58,12 @@ struct Sp16L2 : Sp16<Tr> {
         for (int q = 0; q < 3; ++q) {
             const uint4 w = __ldcg(p + q * vh + i);
             const float2 a = Tr::to_f2(w.x), b = Tr::to_f2(w.y), c = Tr::to_f2(w.z), d = Tr::to_f2(w.w);
-            v[4 * q + 0] = {R(a.x * n), R(a.y * n)};
-            v[4 * q + 1] = {R(b.x * n), R(b.y * n)};
-            v[4 * q + 2] = {R(c.x * n), R(c.y * n)};
-            v[4 * q + 3] = {R(d.x * n), R(d.y * n)};
+            v[4 * q + 0] = {R(a.x), R(a.y)};
+            v[4 * q + 1] = {R(b.x), R(b.y)};
+            v[4 * q + 2] = {R(c.x), R(c.y)};
+            v[4 * q + 3] = {R(d.x), R(d.y)};
         }
+        return n;
     }
 };
 

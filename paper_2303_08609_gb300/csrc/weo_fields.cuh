@@ -23,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace weo {
 
 template <typename T>
@@ -162,21 +164,49 @@ struct LdL2 {
     __device__ static __forceinline__ T ld(const T *p) { return __ldcg(p); }
 };
 
+// Element i of a plane. With a 32-bit index the byte offset is formed in 32
+// bits, so that a load is one instruction on a warp-uniform base (callers
+// guarantee i * sizeof(T) < 2^32); with a 64-bit index it is ordinary pointer
+// arithmetic.
+template <typename T, typename I>
+__device__ __forceinline__ const T *at(const T *plane, I i)
+{
+    if constexpr (std::is_same<I, uint32_t>::value)
+        return reinterpret_cast<const T *>(reinterpret_cast<const char *>(plane) + i * (uint32_t)sizeof(T));
+    else
+        return plane + i;
+}
+
 // ---------------------------------------------------------------- spinors --
+// load() returns the factor that the values still need: none, or the site's norm
+// of the 16-bit formats. The hops apply it to the projected spinor (scale_rows),
+// 12 values instead of 24, with a multiplication that cannot be contracted into
+// the projection's additions, so every kernel rounds alike.
+struct NoScale {};
+
+template <typename R>
+__device__ __forceinline__ void scale_rows(cx<R> (&)[2][3], NoScale) {}
+__device__ __forceinline__ void scale_rows(cx<float> (&h)[2][3], float n)
+{
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        h[k / 3][k % 3] = {__fmul_rn(h[k / 3][k % 3].r, n), __fmul_rn(h[k / 3][k % 3].i, n)};
+}
 
 struct SpF64 {
     using real = double;
     static constexpr int kBytesPerSite = 192;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ NoScale load(const void *base, long long vh, I i,
                                                 cx<R> v[12])
     {
         const double2 *p = static_cast<const double2 *>(base);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            double2 d = ld_keep(p + k * vh + i);
+            double2 d = ld_keep(at(p + k * vh, i));
             v[k] = {R(d.x), R(d.y)};
         }
+        return NoScale();
     }
     template <typename R>
     __device__ static __forceinline__ void store(void *base, long long vh, long long i,
@@ -191,16 +221,17 @@ struct SpF64 {
 struct SpF32 {
     using real = float;
     static constexpr int kBytesPerSite = 96;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ NoScale load(const void *base, long long vh, I i,
                                                 cx<R> v[12])
     {
         const float2 *p = static_cast<const float2 *>(base);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            float2 d = ld_keep(p + k * vh + i);
+            float2 d = ld_keep(at(p + k * vh, i));
             v[k] = {R(d.x), R(d.y)};
         }
+        return NoScale();
     }
     template <typename R>
     __device__ static __forceinline__ void store(void *base, long long vh, long long i,
@@ -218,7 +249,7 @@ struct SpFF {
     using real = ff;
     static constexpr int kBytesPerSite = 192;
     template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    __device__ static __forceinline__ NoScale load(const void *base, long long vh, long long i,
                                                 cx<R> v[12])
     {
         const float2 *p = static_cast<const float2 *>(base);
@@ -227,6 +258,7 @@ struct SpFF {
             const float2 h = ld_keep(p + k * vh + i), l = ld_keep(p + (12 + k) * vh + i);
             v[k] = {ff(h.x, l.x), ff(h.y, l.y)};
         }
+        return NoScale();
     }
     __device__ static __forceinline__ void store(void *base, long long vh, long long i, const cx<ff> v[12])
     {
@@ -272,22 +304,23 @@ template <class Tr>
 struct Sp16 {
     using real = float;
     static constexpr int kBytesPerSite = 52;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ float load(const void *base, long long vh, I i,
                                                 cx<R> v[12])
     {
         const uint4 *p = static_cast<const uint4 *>(base);
         const float *nrm = reinterpret_cast<const float *>(p + 3 * vh);
-        const float n = ld_keep(nrm + i);
+        const float n = ld_keep(at(nrm, i));
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            uint4 w = ld_keep(p + q * vh + i);
+            uint4 w = ld_keep(at(p + q * vh, i));
             float2 a = Tr::to_f2(w.x), b = Tr::to_f2(w.y), c = Tr::to_f2(w.z), d = Tr::to_f2(w.w);
-            v[4 * q + 0] = {R(a.x * n), R(a.y * n)};
-            v[4 * q + 1] = {R(b.x * n), R(b.y * n)};
-            v[4 * q + 2] = {R(c.x * n), R(c.y * n)};
-            v[4 * q + 3] = {R(d.x * n), R(d.y * n)};
+            v[4 * q + 0] = {R(a.x), R(a.y)};
+            v[4 * q + 1] = {R(b.x), R(b.y)};
+            v[4 * q + 2] = {R(c.x), R(c.y)};
+            v[4 * q + 3] = {R(d.x), R(d.y)};
         }
+        return n;
     }
     template <typename R>
     __device__ static __forceinline__ void store(void *base, long long vh, long long i,
@@ -316,25 +349,36 @@ using SpB16 = Sp16<B16Traits>;
 
 // ------------------------------------------------------------------ links --
 
+// conj(a b - c d) in eight operations, none of which the compiler may contract
+// in another way (every kernel rounds alike)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename R>
+__device__ __forceinline__ cx<R> cross_conj(cx<R> a, cx<R> b, cx<R> c, cx<R> d)
+{
+    return {fma(c.i, d.i, fma(-c.r, d.r, fma(-a.i, b.i, mul_rn(a.r, b.r)))),
+            fma(c.i, d.r, fma(c.r, d.i, fma(-a.i, b.r, mul_rn(-a.r, b.i))))};
+}
+
 template <typename R>
 __device__ __forceinline__ void reconstruct_row2(cx<R> U[3][3])
 {
     // row2 = conj(row0 x row1), exact for SU(3)
-    U[2][0] = cconj(csub(cmul(U[0][1], U[1][2]), cmul(U[0][2], U[1][1])));
-    U[2][1] = cconj(csub(cmul(U[0][2], U[1][0]), cmul(U[0][0], U[1][2])));
-    U[2][2] = cconj(csub(cmul(U[0][0], U[1][1]), cmul(U[0][1], U[1][0])));
+    U[2][0] = cross_conj(U[0][1], U[1][2], U[0][2], U[1][1]);
+    U[2][1] = cross_conj(U[0][2], U[1][0], U[0][0], U[1][2]);
+    U[2][2] = cross_conj(U[0][0], U[1][1], U[0][1], U[1][0]);
 }
 
 struct LkF64_18 {
     static constexpr int kBytesPerSite = 144;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ void load(const void *base, long long vh, I i,
                                                 cx<R> U[3][3])
     {
         const double2 *p = static_cast<const double2 *>(base);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            double2 d = ld_stream(p + k * vh + i);
+            double2 d = ld_stream(at(p + k * vh, i));
             U[k / 3][k % 3] = {R(d.x), R(d.y)};
         }
     }
@@ -349,14 +393,14 @@ struct LkF64_18 {
 
 struct LkF64_12 {
     static constexpr int kBytesPerSite = 96;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ void load(const void *base, long long vh, I i,
                                                 cx<R> U[3][3])
     {
         const double2 *p = static_cast<const double2 *>(base);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            double2 d = ld_stream(p + k * vh + i);
+            double2 d = ld_stream(at(p + k * vh, i));
             U[k / 3][k % 3] = {R(d.x), R(d.y)};
         }
         reconstruct_row2(U);
@@ -373,14 +417,14 @@ struct LkF64_12 {
 template <class Ld = LdStream>
 struct LkF32_18T {
     static constexpr int kBytesPerSite = 72;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ void load(const void *base, long long vh, I i,
                                                 cx<R> U[3][3])
     {
         const float4 *p = static_cast<const float4 *>(base);
-        float4 a = Ld::ld(p + i), b = Ld::ld(p + vh + i), c = Ld::ld(p + 2 * vh + i),
-               d = Ld::ld(p + 3 * vh + i);
-        float2 e = Ld::ld(reinterpret_cast<const float2 *>(p + 4 * vh) + i);
+        float4 a = Ld::ld(at(p, i)), b = Ld::ld(at(p + vh, i)), c = Ld::ld(at(p + 2 * vh, i)),
+               d = Ld::ld(at(p + 3 * vh, i));
+        float2 e = Ld::ld(at(reinterpret_cast<const float2 *>(p + 4 * vh), i));
         U[0][0] = {R(a.x), R(a.y)};
         U[0][1] = {R(a.z), R(a.w)};
         U[0][2] = {R(b.x), R(b.y)};
@@ -406,12 +450,12 @@ struct LkF32_18T {
 template <class Ld = LdStream>
 struct LkF32_12T {
     static constexpr int kBytesPerSite = 48;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ void load(const void *base, long long vh, I i,
                                                 cx<R> U[3][3])
     {
         const float4 *p = static_cast<const float4 *>(base);
-        float4 a = Ld::ld(p + i), b = Ld::ld(p + vh + i), c = Ld::ld(p + 2 * vh + i);
+        float4 a = Ld::ld(at(p, i)), b = Ld::ld(at(p + vh, i)), c = Ld::ld(at(p + 2 * vh, i));
         U[0][0] = {R(a.x), R(a.y)};
         U[0][1] = {R(a.z), R(a.w)};
         U[0][2] = {R(b.x), R(b.y)};
@@ -433,13 +477,13 @@ struct LkF32_12T {
 template <class Tr, class Ld = LdStream>
 struct Lk16_18 {
     static constexpr int kBytesPerSite = 36;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ void load(const void *base, long long vh, I i,
                                                 cx<R> U[3][3])
     {
         const uint4 *p = static_cast<const uint4 *>(base);
-        uint4 a = Ld::ld(p + i), b = Ld::ld(p + vh + i);
-        uint32_t e = Ld::ld(reinterpret_cast<const unsigned int *>(p + 2 * vh) + i);
+        uint4 a = Ld::ld(at(p, i)), b = Ld::ld(at(p + vh, i));
+        uint32_t e = Ld::ld(at(reinterpret_cast<const unsigned int *>(p + 2 * vh), i));
         const uint32_t w[9] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, e};
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
@@ -463,13 +507,13 @@ struct Lk16_18 {
 template <class Tr, class Ld = LdStream>
 struct Lk16_12 {
     static constexpr int kBytesPerSite = 24;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
+    template <typename R, typename I>
+    __device__ static __forceinline__ void load(const void *base, long long vh, I i,
                                                 cx<R> U[3][3])
     {
         const uint4 *p = static_cast<const uint4 *>(base);
-        uint4 a = Ld::ld(p + i);
-        uint2 b = Ld::ld(reinterpret_cast<const uint2 *>(p + vh) + i);
+        uint4 a = Ld::ld(at(p, i));
+        uint2 b = Ld::ld(at(reinterpret_cast<const uint2 *>(p + vh), i));
         const uint32_t w[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
