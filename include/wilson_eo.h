@@ -445,7 +445,7 @@ int wilson_eo_get_tile_links(wilson_eo_t h, int *groups, int *rhs_per_thread);
  * links come from the handle's canonical gauge field, split into float-float
  * once (4V x 144 bytes, kept until set_gauge). in_e / out_e: nrhs canonical
  * complex128 even spinors (host or device, as for wilson_eo_apply); the
- * handle keeps three float-float work fields of the same size. Same errors
+ * handle keeps two float-float work fields of the same size. Same errors
  * as wilson_eo_apply. */
 int wilson_eo_apply_ff64(wilson_eo_t h, void *out_e, const void *in_e, int nrhs, int dag, void *stream);
 

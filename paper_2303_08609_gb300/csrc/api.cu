@@ -170,7 +170,7 @@ int handle_hop(wilson_eo_s *h, int prec, int fmt, int io, bool dag, bool axpy, c
 // operators read and write spinors of their own precision; 16-bit operators
 // read and write FP32 spinors and keep the intermediate in 16-bit.
 int meo_with(wilson_eo_s *h, const PackedGauge &g, Buffer &tmp, void *out, const void *in,
-             int nrhs, bool dag, cudaStream_t s)
+             int nrhs, bool dag, cudaStream_t s, bool out_f64)
 {
     const int prec = g.prec;
     if (h->algo == 2 && prec == WEO_F32 && g.fmt == WEO_LINK18) {
@@ -193,6 +193,7 @@ int meo_with(wilson_eo_s *h, const PackedGauge &g, Buffer &tmp, void *out, const
     p.nrhs = nrhs;
     p.gauge = static_cast<const char *>(g.buf.ptr);
     p.gauge_pb = g.pb;
+    p.out_f64 = out_f64;
     const long long ext = h->vh * (prec == WEO_F64 || prec == kPrecFF ? 192 : 96);
     if (prec == WEO_F64 || prec == WEO_F32 || prec == kPrecFF) {
         WEO_TRY(tmp.ensure((size_t)ext * nrhs));
@@ -271,10 +272,8 @@ static int apply_ff_common(wilson_eo_t h, void *out_e, const void *in_e, int nrh
     const PackedGauge *gf = nullptr;
     WEO_TRY(ff_gauge(h, &gf, s));
     WEO_TRY(h->ff_in.ensure(bytes));
-    WEO_TRY(h->ff_out.ensure(bytes));
     WEO_TRY(ff_from_f64(h->ff_in.ptr, in, h->vh, nrhs, s));
-    WEO_TRY(meo_with(h, *gf, h->ff_tmp, h->ff_out.ptr, h->ff_in.ptr, nrhs, dag, s));
-    WEO_TRY(ff_to_f64(out, h->ff_out.ptr, h->vh, nrhs, s));
+    WEO_TRY(meo_with(h, *gf, h->ff_tmp, out, h->ff_in.ptr, nrhs, dag, s, true));
     return finish_out(out_e, out, bytes, out_host, s);
 }
 
@@ -563,7 +562,7 @@ int wilson_eo_info(wilson_eo_t h, int dims_out[4], long long *half_volume, int *
     if (kappa) *kappa = h->kappa;
     if (device_bytes)
         *device_bytes = h->gauge.buf.bytes + h->gauge_f64.buf.bytes + h->gauge_lo.buf.bytes +
-                        h->gauge_ff.buf.bytes + h->ff_in.bytes + h->ff_out.bytes + h->ff_tmp.bytes +
+                        h->gauge_ff.buf.bytes + h->ff_in.bytes + h->ff_tmp.bytes +
                         h->canon_gauge.bytes + h->tmp.bytes + h->tmp2.bytes + h->tmp3.bytes +
                         h->even1.bytes + h->fused_ctrl.bytes + h->halo.bytes + h->staged_links.bytes + h->fs_links.bytes +
                         h->stage_in.bytes +
@@ -834,7 +833,6 @@ void wilson_eo_destroy(wilson_eo_t h)
     h->gauge_lo.buf.release();
     h->gauge_ff.buf.release();
     h->ff_in.release();
-    h->ff_out.release();
     h->ff_tmp.release();
     h->canon_gauge.release();
     h->tmp.release();

@@ -4,51 +4,33 @@
 
 namespace weo {
 
-// src: nrhs x [12][vh] double2 ; dst: nrhs x ([12][vh] float2 high parts, [12][vh] low parts)
-__global__ void k_f64_to_ff(float2 *__restrict__ dst, const double2 *__restrict__ src, long long vh,
-                            long long n)
+// src: nrhs x [12][vh] double2 ; dst: nrhs x ([12][vh] float2 high parts, [12][vh] low parts).
+// One right-hand side per blockIdx.y; ff_split keeps it off the FP64 pipe.
+constexpr int kSplitPer = 4;  // values per thread, all loads in flight together
+__global__ void __launch_bounds__(256) k_f64_to_ff(float2 *__restrict__ dst, const double2 *__restrict__ src, long long per)
 {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long per = 12 * vh, r = e / per, k = e - r * per;
-        const double2 v = src[e];
-        const float hx = float(v.x), hy = float(v.y);
-        float2 *d = dst + r * 2 * per + k;
-        d[0] = make_float2(hx, hy);
-        d[per] = make_float2(float(v.x - double(hx)), float(v.y - double(hy)));
+    const long long k0 = blockIdx.x * (256ll * kSplitPer) + threadIdx.x;
+    const double2 *s = src + blockIdx.y * per;
+    float2 *d = dst + blockIdx.y * 2 * per;
+    double2 v[kSplitPer];
+#pragma unroll
+    for (int j = 0; j < kSplitPer; ++j)
+        if (k0 + 256 * j < per) v[j] = __ldcs(s + k0 + 256 * j);
+#pragma unroll
+    for (int j = 0; j < kSplitPer; ++j) {
+        const long long k = k0 + 256 * j;
+        if (k >= per) break;
+        const float2 a = ff_split(v[j].x), b = ff_split(v[j].y);
+        d[k] = make_float2(a.x, b.x);
+        d[per + k] = make_float2(a.y, b.y);
     }
-}
-
-__global__ void k_ff_to_f64(double2 *__restrict__ dst, const float2 *__restrict__ src, long long vh,
-                            long long n)
-{
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long per = 12 * vh, r = e / per, k = e - r * per;
-        const float2 *s = src + r * 2 * per + k;
-        const float2 h = s[0], l = s[per];
-        dst[e] = make_double2(double(h.x) + double(l.x), double(h.y) + double(l.y));
-    }
-}
-
-static unsigned conv_grid(long long n)
-{
-    const long long b = (n + 255) / 256;
-    return (unsigned)(b < 1 ? 1 : (b > 65535LL * 16 ? 65535LL * 16 : b));
 }
 
 int ff_from_f64(void *dst, const void *src, long long vh, int nrhs, cudaStream_t s)
 {
-    const long long n = 12 * vh * nrhs;
-    k_f64_to_ff<<<conv_grid(n), 256, 0, s>>>(static_cast<float2 *>(dst), static_cast<const double2 *>(src), vh, n);
-    WEO_CUDA(cudaGetLastError());
-    return WEO_OK;
-}
-
-int ff_to_f64(void *dst, const void *src, long long vh, int nrhs, cudaStream_t s)
-{
-    const long long n = 12 * vh * nrhs;
-    k_ff_to_f64<<<conv_grid(n), 256, 0, s>>>(static_cast<double2 *>(dst), static_cast<const float2 *>(src), vh, n);
+    const long long per = 12 * vh;
+    const dim3 grid((unsigned)((per + 256 * kSplitPer - 1) / (256 * kSplitPer)), (unsigned)nrhs);
+    k_f64_to_ff<<<grid, 256, 0, s>>>(static_cast<float2 *>(dst), static_cast<const double2 *>(src), per);
     WEO_CUDA(cudaGetLastError());
     return WEO_OK;
 }

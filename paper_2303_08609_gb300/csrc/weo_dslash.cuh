@@ -69,6 +69,7 @@ struct HopParams {
     long long gauge_pb;
     double a;              // axpy coefficient
     int reverse;           // walk the sites from the top (blocks in reverse order)
+    int out_f64;           // float-float operator: write complex128 (with the axpy only)
     int blocked;           // CTAs take 2x2x2 blocks of rows in (y, z, t) (blockDim = 8 Lx/2)
 };
 
@@ -114,6 +115,21 @@ __device__ __forceinline__ void reconstruct(cx<R> &o0, cx<R> &o1, cx<R> &o2, cx<
     }
 }
 
+// chi = W h for the two spin rows: W = U (FWD) or U^dag
+template <bool FWD, typename T>
+__device__ __forceinline__ void link_mul(const cx<T> U[3][3], const cx<T> h[2][3], cx<T> w[2][3])
+{
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            cx<T> z = {T(0), T(0)};
+#pragma unroll
+            for (int b = 0; b < 3; ++b) z = FWD ? cfma(U[a][b], h[s][b], z) : cfmaconj(U[b][a], h[s][b], z);
+            w[s][a] = z;
+        }
+}
+
 // One hopping direction for R right-hand sides. FWD: link U_mu(x), projector
 // (1 - S0 gamma); backward: link U_mu(x-mu)^dag, projector (1 + S0 gamma).
 template <class SIn, class Lk, int MU, bool FWD, int S0, int R, typename T>
@@ -134,57 +150,11 @@ __device__ __forceinline__ void hop_dir(cx<T> (&acc)[R][12], const HopParams &p,
         for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c]);
         scale_rows(h, n);
         cx<T> w[2][3];
-        if constexpr (std::is_same<T, ff>::value) {
-            // float-float: the six real products of each row are exact and
-            // independent; they are summed pairwise (short dependency chains)
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    ff re[6], im[6];
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) {
-                        const cx<ff> u = FWD ? U[a][b] : U[b][a];
-                        const cx<ff> v = h[s][b];
-                        const ff ui = FWD ? u.i : -u.i;  // conj(u) for the backward hop
-                        re[2 * b] = ff_prod(u.r, v.r);
-                        re[2 * b + 1] = ff_prod(-ui, v.i);
-                        im[2 * b] = ff_prod(u.r, v.i);
-                        im[2 * b + 1] = ff_prod(ui, v.r);
-                    }
-                    w[s][a] = {((re[0] + re[1]) + (re[2] + re[3])) + (re[4] + re[5]),
-                               ((im[0] + im[1]) + (im[2] + im[3])) + (im[4] + im[5])};
-                }
-        } else {
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    cx<T> z = {T(0), T(0)};
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) z = FWD ? cfma(U[a][b], h[s][b], z) : cfmaconj(U[b][a], h[s][b], z);
-                    w[s][a] = z;
-                }
-        }
+        link_mul<FWD>(U, h, w);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
             reconstruct<MU, S>(acc[r][c], acc[r][3 + c], acc[r][6 + c], acc[r][9 + c], w[0][c], w[1][c]);
     }
-}
-
-// chi = W h for the two spin rows: W = U (FWD) or U^dag
-template <bool FWD, typename T>
-__device__ __forceinline__ void link_mul(const cx<T> U[3][3], const cx<T> h[2][3], cx<T> w[2][3])
-{
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            cx<T> z = {T(0), T(0)};
-#pragma unroll
-            for (int b = 0; b < 3; ++b) z = FWD ? cfma(U[a][b], h[s][b], z) : cfmaconj(U[b][a], h[s][b], z);
-            w[s][a] = z;
-        }
 }
 
 // The forward and backward hop of direction MU together (FP64, whose pipe

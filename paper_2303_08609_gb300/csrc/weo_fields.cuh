@@ -34,75 +34,44 @@ struct cx {
 
 // ---------------------------------------------------------- float-float --
 // A float-float number hi + lo (|lo| <= half an ulp of hi) carries about 48
-// significant bits, enough for FP64-class accuracy, with FP32 arithmetic only:
-// Knuth's error-free two-sum, the FMA-based exact product of two floats
-// (Dekker's product without splitting) and the usual renormalisation
-// (double-float arithmetic as in Dekker 1971 and the QD / DSFUN libraries).
-// On GB300 the FP32 pipes issue 64 times as many operations per cycle as the
-// FP64 pipe, so a stencil in this arithmetic outruns native FP64 several-fold.
-// The _rn intrinsics keep the compiler from contracting the error-free steps
-// into fused multiply-adds, which would change what they compute.
+// significant bits, enough for FP64-class accuracy, with FP32 arithmetic only
+// (double-float arithmetic as in Dekker 1971). On GB300 the FP32 pipes issue 64
+// times as many operations per cycle as the FP64 pipe.
 struct ff {
     float hi, lo;
     ff() = default;
-    __host__ __device__ constexpr ff(float h, float l) : hi(h), lo(l) {}
-    __host__ __device__ constexpr ff(int v) : hi(float(v)), lo(0.f) {}
-    __host__ __device__ constexpr ff(float v) : hi(v), lo(0.f) {}
-    __device__ ff(double v) : hi(float(v)), lo(float(v - double(float(v)))) {}
+    __device__ explicit ff(double v) : hi(float(v)), lo(float(v - double(float(v)))) {}
 };
 
-// s + e = a + b exactly
-__device__ __forceinline__ void ff_two_sum(float a, float b, float &s, float &e)
+// hi + lo as a double, correctly rounded, by integer arithmetic (conversions and
+// additions of doubles would run on the FP64 pipe, at 1/64 of the FP32 rate); out
+// of the range of the scale factor, and for infinities and NaN, by the FP64 pipe
+__device__ __forceinline__ double ff_join(float hi, float lo)
 {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-// s + e = a + b exactly, given |a| >= |b| (or a = 0)
-__device__ __forceinline__ void ff_fast_two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    e = __fsub_rn(b, __fsub_rn(s, a));
-}
-
-__device__ __forceinline__ ff operator-(ff a) { return ff(-a.hi, -a.lo); }
-__device__ __forceinline__ ff operator+(ff a, ff b)
-{
-    float s, e;
-    ff_two_sum(a.hi, b.hi, s, e);
-    e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-    ff_fast_two_sum(s, e, s, e);
-    return ff(s, e);
-}
-__device__ __forceinline__ ff operator-(ff a, ff b) { return a + (-b); }
-// a * b + (cross terms): exact product of the high parts as (p, e), with the
-// two cross products folded into e (|e| ~ 2^-24 |p|; the sloppy addition
-// below accepts such an unnormalised pair)
-__device__ __forceinline__ ff ff_prod(ff a, ff b)
-{
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return ff(p, e);
+    const uint32_t b = __float_as_uint(hi), E = (b >> 23) & 255u;
+    if (E - 53u > 201u || fabsf(lo) > fabsf(hi)) return double(hi) + double(lo);
+    // lo in units of the result's last place: 2^-52 of hi's binade, or of the one
+    // below when hi is a power of two that lo reduces
+    const uint32_t below = (b & 0x7fffffu) == 0 && (int)(b ^ __float_as_uint(lo)) < 0;
+    const int L = __float2int_rn(lo * __uint_as_float((306u - E + below) << 23));
+    const long long m = (((long long)(b & 0x7fffffffu) + (896ll << 23)) << 29) + ((int)b < 0 ? -L : L);
+    return __longlong_as_double(m | ((long long)(b & 0x80000000u) << 32));
 }
 
-// the float and double fma stay visible next to the float-float one
-using ::fma;
-
-// c + a * b: exact product of the high parts, cross terms in FP32, one
-// renormalised sum
-__device__ __forceinline__ ff fma(ff a, ff b, ff c)
+// d as hi + lo, the inverse of ff_join
+__device__ __forceinline__ float2 ff_split(double d)
 {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    float s, t;
-    ff_two_sum(p, c.hi, s, t);
-    t = __fadd_rn(t, __fadd_rn(e, c.lo));
-    ff_fast_two_sum(s, t, s, t);
-    return ff(s, t);
+    const long long x = __double_as_longlong(d), a = x & 0x7fffffffffffffffll;
+    const uint32_t E = (uint32_t)(a >> 52);
+    if (E - 950u > 190u) {  // outside 2^-73 .. 2^117
+        const float h = float(d);
+        return make_float2(h, float(d - double(h)));
+    }
+    const long long hi = (a + (1ll << 28)) >> 29;  // rounded to 24 bits, exponent + 896
+    const int r = (int)(a - (hi << 29));           // remainder in units of d's 2^-52
+    const uint32_t s = (uint32_t)(x >> 32) & 0x80000000u;
+    const float lo = __int2float_rn(r) * __uint_as_float((E - 948u) << 23);
+    return make_float2(__uint_as_float((uint32_t)(hi - (896ll << 23)) | s), __uint_as_float(__float_as_uint(lo) ^ s));
 }
 
 template <typename T>
@@ -240,34 +209,6 @@ struct SpF32 {
         float2 *p = static_cast<float2 *>(base);
 #pragma unroll
         for (int k = 0; k < 12; ++k) p[k * vh + i] = make_float2(float(v[k].r), float(v[k].i));
-    }
-};
-
-// FP64-class spinor in float-float: 12 planes of the high parts, then 12 of
-// the low parts (192 bytes per site, as FP64).
-struct SpFF {
-    using real = ff;
-    static constexpr int kBytesPerSite = 192;
-    template <typename R>
-    __device__ static __forceinline__ NoScale load(const void *base, long long vh, long long i,
-                                                cx<R> v[12])
-    {
-        const float2 *p = static_cast<const float2 *>(base);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const float2 h = ld_keep(p + k * vh + i), l = ld_keep(p + (12 + k) * vh + i);
-            v[k] = {ff(h.x, l.x), ff(h.y, l.y)};
-        }
-        return NoScale();
-    }
-    __device__ static __forceinline__ void store(void *base, long long vh, long long i, const cx<ff> v[12])
-    {
-        float2 *p = static_cast<float2 *>(base);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            p[k * vh + i] = make_float2(v[k].r.hi, v[k].i.hi);
-            p[(12 + k) * vh + i] = make_float2(v[k].r.lo, v[k].i.lo);
-        }
     }
 };
 
@@ -538,18 +479,6 @@ struct Lk16_12 {
 // then the low parts in the same layout (144 bytes per site, as FP64).
 struct LkFF18 {
     static constexpr int kBytesPerSite = 144;
-    template <typename R>
-    __device__ static __forceinline__ void load(const void *base, long long vh, long long i,
-                                                cx<R> U[3][3])
-    {
-        cx<float> H[3][3], L[3][3];
-        LkF32_18T<>::load(base, vh, i, H);
-        LkF32_18T<>::load(static_cast<const char *>(base) + 72 * vh, vh, i, L);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) U[a][b] = {ff(H[a][b].r, L[a][b].r), ff(H[a][b].i, L[a][b].i)};
-    }
     __device__ static __forceinline__ void store(void *base, long long vh, long long i,
                                                  const cx<double> U[3][3])
     {

@@ -97,7 +97,7 @@ struct wilson_eo_s {
     weo::PackedGauge gauge_f64;  // solver: true residual (lazy)
     weo::PackedGauge gauge_lo;   // solver: inner operator of an FP64 handle (lazy)
     weo::PackedGauge gauge_ff;   // float-float operator (lazy)
-    weo::Buffer ff_in, ff_out, ff_tmp;  // float-float spinors of wilson_eo_apply_ff64
+    weo::Buffer ff_in, ff_tmp;   // float-float spinors of wilson_eo_apply_ff64
     weo::Buffer canon_gauge;     // device copy of the canonical field (kept for lazy packs)
     int canon_is_f64 = 1;
     weo::Buffer tmp;             // odd-site intermediate of M_eo
@@ -186,9 +186,10 @@ int handle_hop(wilson_eo_s *h, int prec, int fmt, int io, bool dag, bool axpy, c
                cudaStream_t s);
 
 // M_eo / M_eo^dag with a given packed gauge field (its precision decides the
-// spinor formats) and odd-site buffer (api.cu)
+// spinor formats) and odd-site buffer (api.cu); out_f64: the float-float operator
+// writes complex128 instead of SpFF
 int meo_with(wilson_eo_s *h, const PackedGauge &g, Buffer &tmp, void *out, const void *in,
-             int nrhs, bool dag, cudaStream_t s);
+             int nrhs, bool dag, cudaStream_t s, bool out_f64 = false);
 // fused.cu: both hops in one persistent launch over a wavefront of t-slices
 // (FP32 spinors, odd intermediate in `mid`); error word of its bounded waits
 int meo_fused(wilson_eo_s *h, const PackedGauge &g, void *mid, void *out, const void *in, bool dag,
@@ -230,9 +231,8 @@ int solve_full_device(wilson_eo_s *h, void *xi_e, void *xi_o, const void *eta_e,
                       int *iters_out, double *relres_out, cudaStream_t user);
 
 // Pack a canonical gauge field (device memory) into `g` (allocates).
-// ff.cu: complex128 <-> float-float spinors (nrhs x V/2 sites), float-float gauge
+// ff.cu: complex128 -> float-float spinors (nrhs x V/2 sites), float-float gauge
 int ff_from_f64(void *dst, const void *src, long long vh, int nrhs, cudaStream_t s);
-int ff_to_f64(void *dst, const void *src, long long vh, int nrhs, cudaStream_t s);
 int ff_gauge(wilson_eo_s *h, const PackedGauge **g, cudaStream_t s);
 int pack_gauge(wilson_eo_s *h, PackedGauge &g, int prec, int fmt, const void *canon, int is_f64,
                cudaStream_t s);
