@@ -165,21 +165,20 @@ __device__ __forceinline__ void finish_site(const HopParams &p, char *out, const
     }
 }
 
-// MINB: resident CTAs per SM that the registers are held to
-// MULTI: several right-hand sides, which vary fastest in the grid, so that the
-// CTAs that read the same links run side by side
-template <class SIn, class SOut, class SX, class Lk, bool Dag, bool Axpy, int MINB, bool MULTI>
-__global__ void __launch_bounds__(128, MINB) hop_kernel_dirs(const HopParams p)
+// scratch of one 32-site block
+template <bool OUT16>
+struct DirsShared {
+    float2 chi[8 * 6 * 32];
+    float mx[OUT16 ? 96 : 1];
+    uint32_t wd[OUT16 ? 384 : 1];
+};
+
+// The 32 sites from 32 b on, for right-hand side r, by the 128 threads of a CTA
+template <class SIn, class SOut, class SX, class Lk, bool Dag, bool Axpy, bool MULTI>
+__device__ __forceinline__ void dirs_block(const HopParams &p, int b, int r, DirsShared<Is16<SOut>::value> &sh)
 {
     constexpr int S0 = Dag ? -1 : 1;
-    constexpr bool kOut16 = Is16<SOut>::value;
-    __shared__ float2 chi[8 * 6 * 32];
-    __shared__ float mx[kOut16 ? 96 : 1];
-    __shared__ uint32_t wd[kOut16 ? 384 : 1];
     const int lane = (int)threadIdx.x & 31, w = warp_id();
-    const int r = MULTI ? (int)blockIdx.x % p.nrhs : 0;
-    int b = MULTI ? (int)blockIdx.x / p.nrhs : (int)blockIdx.x;
-    if (p.reverse) b = (MULTI ? (p.vh + 31) / 32 : (int)gridDim.x) - 1 - b;
     const char *in = static_cast<const char *>(p.in) + (MULTI ? r * p.in_stride : 0);
     const int i_raw = b * 32 + lane;
     const bool valid = i_raw < p.vh;
@@ -194,7 +193,7 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel_dirs(const HopParams p)
         const auto n = SIn::load(in, p.vh, nb, v);
         Lk::load(p.gauge + (2 * MU + (FWD ? p.out_parity : p.out_parity ^ 1)) * p.gauge_pb, p.vh,
                  FWD ? (uint32_t)i : nb, U);
-        dir_chi<MU, FWD, S0>(U, v, n, chi + (2 * MU + !FWD) * 192 + lane);
+        dir_chi<MU, FWD, S0>(U, v, n, sh.chi + (2 * MU + !FWD) * 192 + lane);
     };
     auto both = [&](auto mu) {
         dir(mu, std::true_type());
@@ -208,27 +207,37 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel_dirs(const HopParams p)
     }
     float2 xv[4];
     if (Axpy && w < 3) {
-        const float2 *x = reinterpret_cast<const float2 *>(static_cast<const char *>(p.x) + (MULTI ? r * p.x_stride : 0)) + (long long)w * p.vh;
+        const float2 *x = reinterpret_cast<const float2 *>(static_cast<const char *>(p.x) + (MULTI ? r * p.x_stride : 0)) +
+                          (long long)w * p.vh;
 #pragma unroll
         for (int k = 0; k < 4; ++k) xv[k] = ld_keep(at(x + 3ll * k * p.vh, (uint32_t)i));
     }
     __syncthreads();
     if (w < 3)
-        finish_site<SOut, Dag, Axpy>(p, static_cast<char *>(p.out) + (MULTI ? r * p.out_stride : 0), chi + 32 * w + lane,
-                                     w, lane, (uint32_t)i, valid, xv, mx, wd);
+        finish_site<SOut, Dag, Axpy>(p, static_cast<char *>(p.out) + (MULTI ? r * p.out_stride : 0),
+                                     sh.chi + 32 * w + lane, w, lane, (uint32_t)i, valid, xv, sh.mx, sh.wd);
+}
+
+// MINB: resident CTAs per SM that the registers are held to
+// MULTI: several right-hand sides, which vary fastest in the grid, so that the
+// CTAs that read the same links run side by side
+template <class SIn, class SOut, class SX, class Lk, bool Dag, bool Axpy, int MINB, bool MULTI>
+__global__ void __launch_bounds__(128, MINB) hop_kernel_dirs(const HopParams p)
+{
+    __shared__ DirsShared<Is16<SOut>::value> sh;
+    const int r = MULTI ? (int)blockIdx.x % p.nrhs : 0;
+    int b = MULTI ? (int)blockIdx.x / p.nrhs : (int)blockIdx.x;
+    if (p.reverse) b = (MULTI ? (p.vh + 31) / 32 : (int)gridDim.x) - 1 - b;
+    dirs_block<SIn, SOut, SX, Lk, Dag, Axpy, MULTI>(p, b, r, sh);
 }
 
 // FP64: warp mu of a 128-thread CTA takes the pair of directions +-mu of 32
 // sites (hop_pair); three warps then add the four pairs, one colour each.
 template <class Lk, bool Dag, bool Axpy>
-__global__ void __launch_bounds__(128, 3) hop_kernel_pairs(const HopParams p)
+__device__ __forceinline__ void pairs_block(const HopParams &p, int b, int r, double2 *part)
 {
     constexpr int S0 = Dag ? -1 : 1;
-    __shared__ double2 part[4 * 12 * 32];
     const int lane = (int)threadIdx.x & 31, w = warp_id();
-    const int r = (int)blockIdx.x % p.nrhs;
-    int b = (int)blockIdx.x / p.nrhs;
-    if (p.reverse) b = (p.vh + 31) / 32 - 1 - b;
     const int i_raw = b * 32 + lane;
     const bool valid = i_raw < p.vh;
     const int i = valid ? i_raw : p.vh - 1;
@@ -284,6 +293,16 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pairs(const HopParams p)
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         *const_cast<double2 *>(at(q + 3ll * k * p.vh, (uint32_t)i)) = make_double2(o[k].r, o[k].i);
+}
+
+template <class Lk, bool Dag, bool Axpy>
+__global__ void __launch_bounds__(128, 3) hop_kernel_pairs(const HopParams p)
+{
+    __shared__ double2 part[4 * 12 * 32];
+    const int r = (int)blockIdx.x % p.nrhs;
+    int b = (int)blockIdx.x / p.nrhs;
+    if (p.reverse) b = (p.vh + 31) / 32 - 1 - b;
+    pairs_block<Lk, Dag, Axpy>(p, b, r, part);
 }
 
 // FP64: a 128-thread CTA takes 16 sites; warp mu of it the forward and backward
