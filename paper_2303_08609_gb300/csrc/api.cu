@@ -55,6 +55,17 @@ static bool is_device_pointer(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// memory of GPU `device` itself
+static bool is_memory_of(const void *p, int device)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 // page-locked host memory (cudaHostAlloc / cudaHostRegister / torch pin_memory)
 static bool is_pinned_host_pointer(const void *p)
 {
@@ -132,14 +143,20 @@ static int upload_gauge(wilson_eo_s *h, const void *gauge, int gauge_is_f64, cud
 {
     const size_t bytes = (size_t)(2 * h->vh) * 4 * 9 * (gauge_is_f64 ? 16 : 8);
     WEO_TRY(h->canon_gauge.ensure(bytes));
-    const cudaMemcpyKind kind =
-        is_device_pointer(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    WEO_CUDA(cudaMemcpyAsync(h->canon_gauge.ptr, gauge, bytes, kind, s));
+    // a field in this GPU's memory is copied by the packing kernel that reads it
+    // (one in another GPU's memory is not readable there without peer access)
+    const bool here = is_memory_of(gauge, h->device);
+    if (!here) {
+        const cudaMemcpyKind kind =
+            is_device_pointer(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+        WEO_CUDA(cudaMemcpyAsync(h->canon_gauge.ptr, gauge, bytes, kind, s));
+    }
     h->canon_is_f64 = gauge_is_f64 ? 1 : 0;
     h->gauge_f64.valid = false;
     h->gauge_lo.valid = false;
     h->gauge_ff.valid = false;
-    WEO_TRY(pack_gauge(h, h->gauge, h->prec, h->fmt, h->canon_gauge.ptr, h->canon_is_f64, s));
+    WEO_TRY(pack_gauge(h, h->gauge, h->prec, h->fmt, here ? gauge : h->canon_gauge.ptr, h->canon_is_f64, s,
+                       here ? h->canon_gauge.ptr : nullptr));
     WEO_CUDA(cudaStreamSynchronize(s));
     return WEO_OK;
 }

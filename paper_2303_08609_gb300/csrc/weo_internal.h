@@ -230,11 +230,12 @@ int solve_full_device(wilson_eo_s *h, void *xi_e, void *xi_o, const void *eta_e,
                       const void *eta_o, const bool host[4], double tol, int maxiter, int mixed,
                       int *iters_out, double *relres_out, cudaStream_t user);
 
-// Pack a canonical gauge field (device memory) into `g` (allocates).
 // ff.cu: complex128 -> float-float spinors (nrhs x V/2 sites), float-float gauge
 int ff_from_f64(void *dst, const void *src, long long vh, int nrhs, cudaStream_t s);
 int ff_gauge(wilson_eo_s *h, const PackedGauge **g, cudaStream_t s);
+// Pack a canonical gauge field (device memory) into `g` (allocates); `copy`, if
+// not null, receives a copy of it.
 int pack_gauge(wilson_eo_s *h, PackedGauge &g, int prec, int fmt, const void *canon, int is_f64,
-               cudaStream_t s);
+               cudaStream_t s, void *copy = nullptr);
 
 }  // namespace weo
