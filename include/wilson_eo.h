@@ -136,6 +136,21 @@ int wilson_eo_hop(wilson_eo_t h, int out_parity, int dag, void *out, const void 
 int wilson_eo_link_grad(wilson_eo_t h, void *grad, const void *g_e, const void *phi_e,
                         void *stream);
 
+/* The two halves of a differentiable M_eo, sharing their hops (Eq. 4):
+ *   wilson_eo_grad_forward:  out_e = M_eo in_e, and t_o = H_oe in_e, the odd
+ *                            intermediate, which the backward pass needs
+ *   wilson_eo_grad_backward: for L = Re<g_e, M_eo phi_e>, grad_gauge as in
+ *                            wilson_eo_link_grad with t_o = H_oe phi_e known, and,
+ *                            unless it is NULL, grad_phi = M_eo^dag g_e, whose first
+ *                            hop the link gradient computes anyway
+ * Two hops each instead of two and four. Results equal wilson_eo_apply,
+ * wilson_eo_link_grad and wilson_eo_apply_dag. FP64 / FP32 handles, one right-hand
+ * side, device arrays (WEO_ERR_ARG for host arrays or an output that aliases an
+ * input); asynchronous on `stream`. */
+int wilson_eo_grad_forward(wilson_eo_t h, void *out_e, void *t_o, const void *in_e, void *stream);
+int wilson_eo_grad_backward(wilson_eo_t h, void *grad_phi, void *grad_gauge, const void *g_e,
+                            const void *phi_e, const void *t_o, void *stream);
+
 /* Pseudofermion force of S(U, phi) = |M_eo phi_e|^2 (the Schur-decomposed
  * determinant of Sec. 2 evaluated with a noise vector phi): force[mu][lex] is
  * the traceless anti-Hermitian 3x3 matrix F with dS/d eps = Re tr(X^dag F) for

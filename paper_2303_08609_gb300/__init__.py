@@ -78,6 +78,8 @@ def _load():
     optional = {
         "wilson_eo_force": (I, [P, P, P, P, P]),
         "wilson_eo_link_grad": (I, [P, P, P, P, P]),
+        "wilson_eo_grad_forward": (I, [P, P, P, P, P]),
+        "wilson_eo_grad_backward": (I, [P, P, P, P, P, P, P]),
         "wilson_eo_solve": (I, [P, P, P, D, I, I, IP, ctypes.POINTER(D), P]),
         "wilson_eo_solver_config": (I, [P, D, I, I]),
         "wilson_eo_solve_multi": (I, [P, P, P, I, D, I, I, IP, ctypes.POINTER(D), P]),
@@ -298,6 +300,21 @@ def wilson_eo_link_grad(h, grad, g_e, phi_e, stream=None):
     _expect(h, (grad,), kind="gauge", where="wilson_eo_link_grad")
     _check(_load().wilson_eo_link_grad(h, _ptr(grad), _ptr(g_e), _ptr(phi_e), _stream(stream)),
            "wilson_eo_link_grad")
+
+
+def wilson_eo_grad_forward(h, out_e, t_o, in_e, stream=None):
+    """M_eo in_e, and its odd intermediate H_oe in_e for wilson_eo_grad_backward."""
+    _expect(h, (out_e, t_o, in_e), 1, where="wilson_eo_grad_forward")
+    _check(_load().wilson_eo_grad_forward(h, _ptr(out_e), _ptr(t_o), _ptr(in_e), _stream(stream)),
+           "wilson_eo_grad_forward")
+
+
+def wilson_eo_grad_backward(h, grad_phi, grad_gauge, g_e, phi_e, t_o, stream=None):
+    """Link gradient of Re<g, M_eo phi>, and M_eo^dag g unless grad_phi is None."""
+    _expect(h, (grad_phi, g_e, phi_e, t_o), 1, where="wilson_eo_grad_backward")
+    _expect(h, (grad_gauge,), kind="gauge", where="wilson_eo_grad_backward")
+    _check(_load().wilson_eo_grad_backward(h, _ptr(grad_phi), _ptr(grad_gauge), _ptr(g_e), _ptr(phi_e),
+                                           _ptr(t_o), _stream(stream)), "wilson_eo_grad_backward")
 
 
 def wilson_eo_force(h, force, dS_dphi_e, phi_e, stream=None):

@@ -14,7 +14,7 @@ from __future__ import annotations
 
 import torch
 
-from . import WilsonEO
+from . import WilsonEO, wilson_eo_grad_backward, wilson_eo_grad_forward
 
 
 def _sync_gauge(op: WilsonEO, U: torch.Tensor, refresh):
@@ -44,16 +44,29 @@ class MeoFunction(torch.autograd.Function):
         phi = phi.contiguous()
         ctx.op = op
         ctx.refresh = refresh
-        ctx.save_for_backward(phi, U)
-        return op.apply(phi)
+        if not ctx.needs_input_grad[1] or phi.dim() != 3 or not phi.is_cuda:
+            ctx.save_for_backward(phi, U)
+            return op.apply(phi)
+        # the link gradient needs the odd intermediate: keep it, one spinor, rather
+        # than spend a third hop on it in the backward pass
+        op._nrhs(phi)
+        out, t = torch.empty_like(phi), torch.empty_like(phi)
+        wilson_eo_grad_forward(op.handle, out, t, phi)
+        ctx.save_for_backward(phi, U, t)
+        return out
 
     @staticmethod
     def backward(ctx, grad_out):
-        phi, U = ctx.saved_tensors
+        phi, U, *mid = ctx.saved_tensors
         op = ctx.op
         # the handle may hold another forward's links by now
         _sync_gauge(op, U, ctx.refresh)
         g = grad_out.contiguous()
+        if ctx.needs_input_grad[1] and mid:
+            grad_phi = torch.empty_like(phi) if ctx.needs_input_grad[0] else None
+            grad_U = torch.empty((4, 2 * op.vh, 3, 3), dtype=op.spinor_dtype(), device=phi.device)
+            wilson_eo_grad_backward(op.handle, grad_phi, grad_U, g, phi, mid[0])
+            return grad_phi, grad_U, None, None
         grad_phi = op.apply(g, dag=True) if ctx.needs_input_grad[0] else None
         grad_U = None
         if ctx.needs_input_grad[1]:

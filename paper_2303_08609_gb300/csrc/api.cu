@@ -254,6 +254,22 @@ int meo_device(wilson_eo_s *h, void *out, const void *in, int nrhs, bool dag, cu
     return meo_with(h, h->gauge, h->tmp, out, in, nrhs, dag, s);
 }
 
+int meo_second_hop(wilson_eo_s *h, void *out, const void *x, const void *mid, bool dag, cudaStream_t s)
+{
+    HopParams p = geom_params(h);
+    p.nrhs = 1;
+    p.gauge = static_cast<const char *>(h->gauge.buf.ptr);
+    p.gauge_pb = h->gauge.pb;
+    p.in_stride = p.out_stride = p.x_stride = (long long)ext_spinor_bytes(h);
+    p.out_parity = 0;
+    p.in = mid;
+    p.out = out;
+    p.x = x;
+    p.a = -h->kappa * h->kappa;
+    p.reverse = h->alternate;
+    return handle_hop(h, h->prec, h->fmt, IO_SAME, dag, true, p, s);
+}
+
 static int apply_common(wilson_eo_t h, void *out_e, const void *in_e, int nrhs, bool dag,
                         void *stream)
 {
@@ -685,11 +701,53 @@ int wilson_eo_force(wilson_eo_t h, void *force, void *dS_dphi_e, const void *phi
         WEO_TRY(meo_device(h, h->even1.ptr, phi, 1, false, s));
         WEO_TRY(scale_spinor(h, h->even1.ptr, 1, 2.0, s));
         WEO_TRY(link_grad_device(h, out, h->even1.ptr, phi, 1, s, h->tmp.ptr));
-        if (dphi) WEO_TRY(meo_device(h, dphi, h->even1.ptr, 1, true, s));  // 2 M^dag M phi
+        // 2 M^dag M phi: its first hop is the w that the gradient left in h->tmp3
+        if (dphi) WEO_TRY(meo_second_hop(h, dphi, h->even1.ptr, h->tmp3.ptr, true, s));
         if (dphi) WEO_TRY(finish_out(dS_dphi_e, dphi, sb, dphi_host, s));
         return finish_out(force, out, gb, out_host, s);
     } catch (...) {
         return set_error(WEO_ERR_OOM, "host exception in wilson_eo_force");
+    }
+}
+
+int wilson_eo_grad_forward(wilson_eo_t h, void *out_e, void *t_o, const void *in_e, void *stream)
+{
+    try {
+        if (!h || !out_e || !t_o || !in_e) return set_error(WEO_ERR_ARG, "NULL handle or array");
+        if (out_e == in_e || t_o == in_e || t_o == out_e) return set_error(WEO_ERR_ARG, "arrays must not alias");
+        if (h->prec != WEO_F64 && h->prec != WEO_F32)
+            return set_error(WEO_ERR_UNSUPPORTED, "the gradient needs an FP64 or FP32 handle");
+        if (!is_device_pointer(out_e) || !is_device_pointer(t_o) || !is_device_pointer(in_e))
+            return set_error(WEO_ERR_ARG, "device arrays only");
+        DeviceGuard dg(h->device);
+        Buffer mid;  // the caller's array in the place of the handle's intermediate
+        mid.ptr = t_o;
+        mid.bytes = ext_spinor_bytes(h);
+        return meo_with(h, h->gauge, mid, out_e, in_e, 1, false, static_cast<cudaStream_t>(stream));
+    } catch (...) {
+        return set_error(WEO_ERR_OOM, "host exception in wilson_eo_grad_forward");
+    }
+}
+
+int wilson_eo_grad_backward(wilson_eo_t h, void *grad_phi, void *grad_gauge, const void *g_e, const void *phi_e,
+                            const void *t_o, void *stream)
+{
+    try {
+        if (!h || !grad_gauge || !g_e || !phi_e || !t_o) return set_error(WEO_ERR_ARG, "NULL handle or array");
+        if (grad_phi && (grad_phi == g_e || grad_phi == phi_e || grad_phi == t_o))
+            return set_error(WEO_ERR_ARG, "grad_phi must not alias an input");
+        if (h->prec != WEO_F64 && h->prec != WEO_F32)
+            return set_error(WEO_ERR_UNSUPPORTED, "the gradient needs an FP64 or FP32 handle");
+        const void *ptrs[4] = {grad_gauge, g_e, phi_e, t_o};
+        for (const void *q : ptrs)
+            if (!is_device_pointer(q)) return set_error(WEO_ERR_ARG, "device arrays only");
+        if (grad_phi && !is_device_pointer(grad_phi)) return set_error(WEO_ERR_ARG, "device arrays only");
+        DeviceGuard dg(h->device);
+        cudaStream_t s = static_cast<cudaStream_t>(stream);
+        WEO_TRY(link_grad_device(h, grad_gauge, g_e, phi_e, 0, s, t_o));
+        return grad_phi ? meo_second_hop(h, grad_phi, g_e, h->tmp3.ptr, true, s) : WEO_OK;
+    } catch (...) {
+        return set_error(WEO_ERR_OOM, "host exception in wilson_eo_grad_backward");
     }
 }
 

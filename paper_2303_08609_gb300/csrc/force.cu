@@ -219,7 +219,7 @@ int link_grad_device(wilson_eo_s *h, void *out, const void *g, const void *phi, 
                      cudaStream_t s, const void *t_known)
 {
     const long long ext = h->vh * (h->prec == WEO_F64 ? 192 : 96);
-    WEO_TRY(h->tmp2.ensure((size_t)ext));
+    if (!t_known) WEO_TRY(h->tmp2.ensure((size_t)ext));
     WEO_TRY(h->tmp3.ensure((size_t)ext));
     HopParams hp = geom_params(h);
     hp.nrhs = 1;

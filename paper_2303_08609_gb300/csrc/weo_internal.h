@@ -208,8 +208,11 @@ int hop_split_device(wilson_eo_s *h, int ranks, int out_parity, bool dag, void *
 // M_eo / M_eo^dag on device arrays in the handle's external format (api.cu)
 int meo_device(wilson_eo_s *h, void *out, const void *in, int nrhs, bool dag, cudaStream_t s);
 // link gradient (force = 0) or force TA(G U^dag) (force = 1), force.cu
+// (t_known: H_oe phi if the caller has it); leaves w = H_eo^dag g in h->tmp3
 int link_grad_device(wilson_eo_s *h, void *out, const void *g, const void *phi, int force,
                      cudaStream_t s, const void *t_known = nullptr);
+// out = x - kappa^2 H_eo^(dag) mid: the second hop of M_eo / M_eo^dag alone (api.cu)
+int meo_second_hop(wilson_eo_s *h, void *out, const void *x, const void *mid, bool dag, cudaStream_t s);
 int scale_spinor(wilson_eo_s *h, void *v, int nrhs, double c, cudaStream_t s);
 
 // solver.cu
