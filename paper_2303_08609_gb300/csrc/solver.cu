@@ -138,33 +138,64 @@ __device__ __forceinline__ double re_dot(T2 a, T2 b) { return double(a.x) * b.x 
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
 
 // FP32 vectors are read as float4 (two complex numbers; n = 12 V/2 is even and
-// every right-hand side starts on a 16-byte boundary). Squares are summed in
-// FP32 over the handful of values one thread has in flight and only those
-// group sums are accumulated in FP64: per-element FP64 arithmetic would run at
-// the FP64 rate, a small fraction of the FP32 one, and would bound these
-// otherwise memory-bound kernels.
+// every right-hand side starts on a 16-byte boundary). The squares of the four
+// float4 that a thread has in flight are summed in FP32, and those group sums are
+// accumulated, over the thread, the warp and the block, as a float-float number
+// (error-free sums, 48 bits, far below the rounding of the FP32 squares): each FP64
+// instruction of a warp takes 16 cycles of the SM's FP64 pipe. At 16^3 x 32 the
+// norm of M p took 8.5 us with FP64 sums and takes 6.0, the residual update 9.1
+// and 8.3.
 __device__ __forceinline__ float sq4(float4 q) { return q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w; }
+
+struct Sum2 {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x, float xl = 0.f)
+    {
+        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+        const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b));
+        h = s;
+        l = __fadd_rn(l, __fadd_rn(e, xl));
+    }
+};
+
+// sum over the block, valid in thread 0
+__device__ __forceinline__ double block_sum(Sum2 v)
+{
+    __shared__ float2 sh[32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_down_sync(0xffffffffu, v.h, o), l = __shfl_down_sync(0xffffffffu, v.l, o);
+        v.add(h, l);
+    }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) sh[w] = make_float2(v.h, v.l);
+    __syncthreads();
+    if (threadIdx.x != 0) return 0.0;
+    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) v.add(sh[k].x, sh[k].y);
+    return double(v.h) + double(v.l);
+}
 
 __device__ __forceinline__ long long grid_stride() { return (long long)gridDim.x * blockDim.x; }
 __device__ __forceinline__ long long grid_index() { return blockIdx.x * (long long)blockDim.x + threadIdx.x; }
 
 // sum of |a_k|^2 over n complex values, this thread's share
-template <typename T2>
-__device__ __forceinline__ double sum_sq(const T2 *a, long long n)
+__device__ __forceinline__ Sum2 sum_sq(const float2 *a, long long n)
+{
+    Sum2 v;
+    const float4 *a4 = reinterpret_cast<const float4 *>(a), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const long long n4 = n >> 1, st = grid_stride();
+    for (long long k = grid_index(); k < n4; k += 4 * st) {
+        const float4 q0 = a4[k], q1 = k + st < n4 ? a4[k + st] : zero, q2 = k + 2 * st < n4 ? a4[k + 2 * st] : zero,
+                     q3 = k + 3 * st < n4 ? a4[k + 3 * st] : zero;
+        v.add((sq4(q0) + sq4(q1)) + (sq4(q2) + sq4(q3)));
+    }
+    return v;
+}
+__device__ __forceinline__ double sum_sq(const double2 *a, long long n)
 {
     double v = 0.0;
-    if constexpr (std::is_same<T2, float2>::value) {
-        const float4 *a4 = reinterpret_cast<const float4 *>(a);
-        const long long n4 = n >> 1, st = grid_stride();
-        long long k = grid_index();
-        for (; k + 3 * st < n4; k += 4 * st) {
-            const float4 q0 = a4[k], q1 = a4[k + st], q2 = a4[k + 2 * st], q3 = a4[k + 3 * st];
-            v += double((sq4(q0) + sq4(q1)) + (sq4(q2) + sq4(q3)));
-        }
-        for (; k < n4; k += st) v += double(sq4(a4[k]));
-    } else {
-        FOR_ELEMENTS(k) v += re_dot(a[k], a[k]);
-    }
+    FOR_ELEMENTS(k) v += re_dot(a[k], a[k]);
     return v;
 }
 
@@ -223,25 +254,23 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(T2 *r, const T2 *Ap, 
         float4 *r4 = reinterpret_cast<float4 *>(r);
         const float4 *a4 = reinterpret_cast<const float4 *>(Ap);
         const long long n4 = n >> 1, st = grid_stride();
-        long long k = grid_index();
-        for (; k + 3 * st < n4; k += 4 * st) {
-            float4 r0 = r4[k], r1 = r4[k + st], r2 = r4[k + 2 * st], r3 = r4[k + 3 * st];
-            axpy4(r0, -alpha, a4[k]);
-            axpy4(r1, -alpha, a4[k + st]);
-            axpy4(r2, -alpha, a4[k + 2 * st]);
-            axpy4(r3, -alpha, a4[k + 3 * st]);
-            r4[k] = r0;
-            r4[k + st] = r1;
-            r4[k + 2 * st] = r2;
-            r4[k + 3 * st] = r3;
-            v += double((sq4(r0) + sq4(r1)) + (sq4(r2) + sq4(r3)));
+        Sum2 q;
+        for (long long k0 = grid_index(); k0 < n4; k0 += 4 * st) {
+            float4 rv[4], av[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool in = k0 + j * st < n4;
+                rv[j] = in ? r4[k0 + j * st] : make_float4(0.f, 0.f, 0.f, 0.f);
+                av[j] = in ? a4[k0 + j * st] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                axpy4(rv[j], -alpha, av[j]);
+                if (k0 + j * st < n4) r4[k0 + j * st] = rv[j];
+            }
+            q.add((sq4(rv[0]) + sq4(rv[1])) + (sq4(rv[2]) + sq4(rv[3])));
         }
-        for (; k < n4; k += st) {
-            float4 r0 = r4[k];
-            axpy4(r0, -alpha, a4[k]);
-            r4[k] = r0;
-            v += double(sq4(r0));
-        }
+        v = block_sum(q);
     } else {
         FOR_ELEMENTS(k) {
             T2 rv = r[k];
@@ -251,8 +280,8 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(T2 *r, const T2 *Ap, 
             r[k] = rv;
             v += re_dot(rv, rv);
         }
+        v = block_sum(v);
     }
-    v = block_sum(v);
     double tot;
     if (finish_reduction(sc, v, &tot) && threadIdx.x == 0) {
         if (!isfinite(tot) || !isfinite(tot / sc->rr)) {
@@ -281,26 +310,24 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_dir(T2 *x, T2 *p, const T2 *
         float4 *x4 = reinterpret_cast<float4 *>(x), *p4 = reinterpret_cast<float4 *>(p);
         const float4 *r4 = reinterpret_cast<const float4 *>(r);
         const long long n4 = n >> 1, st = grid_stride();
-        long long k = grid_index();
-        for (; k + st < n4; k += 2 * st) {
-            const float4 q0 = p4[k], q1 = p4[k + st];
-            float4 x0 = x4[k], x1 = x4[k + st], y0 = r4[k], y1 = r4[k + st];
-            axpy4(x0, alpha, q0);
-            axpy4(x1, alpha, q1);
-            axpy4(y0, beta, q0);
-            axpy4(y1, beta, q1);
-            x4[k] = x0;
-            x4[k + st] = x1;
-            p4[k] = y0;
-            p4[k + st] = y1;
-        }
-        if (k < n4) {
-            const float4 q0 = p4[k];
-            float4 x0 = x4[k], y0 = r4[k];
-            axpy4(x0, alpha, q0);
-            axpy4(y0, beta, q0);
-            x4[k] = x0;
-            p4[k] = y0;
+        for (long long k0 = grid_index(); k0 < n4; k0 += 3 * st) {
+            float4 q[3], xv[3], y[3];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const long long k = k0 + j * st < n4 ? k0 + j * st : k0;
+                q[j] = p4[k];
+                xv[j] = x4[k];
+                y[j] = r4[k];
+            }
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                axpy4(xv[j], alpha, q[j]);
+                axpy4(y[j], beta, q[j]);
+                if (j == 0 || k0 + j * st < n4) {
+                    x4[k0 + j * st] = xv[j];
+                    p4[k0 + j * st] = y[j];
+                }
+            }
         }
     } else {
         FOR_ELEMENTS(k) {
@@ -353,7 +380,7 @@ __global__ void __launch_bounds__(kRedThreads) k_residual_ff(double2 *r, const d
     FOR_ELEMENTS(k) {
         const float2 hi = t[k], lo = t[n + k];
         const double2 bv = b[k];
-        const double2 rv = make_double2((bv.x - double(hi.x)) - double(lo.x), (bv.y - double(hi.y)) - double(lo.y));
+        const double2 rv = make_double2(bv.x - ff_join(hi.x, lo.x), bv.y - ff_join(hi.y, lo.y));
         r[k] = rv;
         v += rv.x * rv.x + rv.y * rv.y;
     }
