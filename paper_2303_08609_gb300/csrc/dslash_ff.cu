@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(128, 4) hop_kernel_ff(const HopParams p)
     constexpr int S0 = Dag ? -1 : 1;
     __shared__ float4 part[4 * 12 * 32];
     const int lane = (int)threadIdx.x & 31, w = warp_id();
+    pdl_wait();
     const int r = (int)blockIdx.y;
     const int b = p.reverse ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x;
     const int i_raw = b * 32 + lane;
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(128, 4) hop_kernel_ff(const HopParams p)
         for (int k = 0; k < 4; ++k) xv[k] = load_fc(x, p.vh, 3 * k + w, (uint32_t)i);
     }
     __syncthreads();
+    pdl_next();
     if (w >= 3 || !valid) return;
     auto read = [&](int m, int k) {
         const float4 q = part[(12 * m + 3 * k + w) * 32 + lane];
@@ -258,9 +260,7 @@ template <bool Dag, bool Axpy, bool OutF64>
 static int launch_ff(const HopParams &p, cudaStream_t s)
 {
     dim3 grid((unsigned)((p.vh + 31) / 32), (unsigned)p.nrhs);
-    hop_kernel_ff<Dag, Axpy, OutF64><<<grid, 128, 0, s>>>(p);
-    WEO_CUDA(cudaGetLastError());
-    return WEO_OK;
+    return launch_dependent(hop_kernel_ff<Dag, Axpy, OutF64>, grid, 128, s, p);
 }
 
 int launch_hop_ff(bool dag, bool axpy, const HopParams &p, const LaunchCfg &, cudaStream_t s)

@@ -73,6 +73,16 @@ struct HopParams {
     int blocked;           // CTAs take 2x2x2 blocks of rows in (y, z, t) (blockDim = 8 Lx/2)
 };
 
+// Programmatic dependent launch: a grid may be placed while its predecessor in the
+// stream still drains. pdl_wait, before the first access to memory, returns when
+// the predecessor has completed and its writes are visible; pdl_next lets the
+// successor's CTAs take the slots that this grid's CTAs leave, once every one of
+// them has reached it. Called when a CTA's loads are done: called first, successors
+// of grids that fill less than a wave were placed beside them and made the next
+// hop uneven (16^4 FP16: 8.6 us per M_eo without, 9.8 early, 7.8 late).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // h = psi_up - S A_mu psi_dn for one colour
 template <int MU, int S, typename R>
 __device__ __forceinline__ void project(const cx<R> p0, const cx<R> p1, const cx<R> p2,

@@ -28,6 +28,24 @@ int fail_cuda(cudaError_t e, const char *what, const char *file, int line);
         if (s_ != WEO_OK) return s_; \
     } while (0)
 
+// Launch as a programmatic dependent of the stream's previous kernel: `kern` starts
+// with pdl_wait. Saves the gap between two kernels, 0.4 to 1 us of each.
+template <typename... K, typename... A>
+int launch_dependent(void (*kern)(K...), dim3 grid, unsigned block, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    WEO_CUDA(cudaLaunchKernelEx(&cfg, kern, K(args)...));
+    return WEO_OK;
+}
+
 // ----------------------------------------------------------------- formats --
 // Internal operator precision next to weo_prec: float-float arithmetic with
 // 18-real links (FP64-class accuracy from FP32 operations); spinors SpFF.

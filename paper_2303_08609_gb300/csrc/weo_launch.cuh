@@ -80,20 +80,16 @@ int launch_split(const HopParams &p, cudaStream_t s)
     const unsigned nsb = (unsigned)((p.vh + 31) / 32);
     if constexpr (std::is_same<typename SOut::real, double>::value) {
         if (p.vh < kRowsMaxSites)
-            hop_kernel_rows<Lk, Dag, Axpy><<<(unsigned)((p.vh + 15) / 16) * p.nrhs, 128, 0, s>>>(p);
-        else
-            hop_kernel_pairs<Lk, Dag, Axpy><<<nsb * p.nrhs, 128, 0, s>>>(p);
+            return launch_dependent(hop_kernel_rows<Lk, Dag, Axpy>, (unsigned)((p.vh + 15) / 16) * p.nrhs, 128, s, p);
+        return launch_dependent(hop_kernel_pairs<Lk, Dag, Axpy>, nsb * p.nrhs, 128, s, p);
     } else {
         constexpr int kMinCtas = Is16<SIn>::value || Is16<SOut>::value ? 10
                                  : std::is_same<Lk, LkF32_12>::value      ? 9
                                                                           : 8;
         if (p.nrhs == 1)
-            hop_kernel_dirs<SIn, SOut, SX, Lk, Dag, Axpy, kMinCtas, false><<<nsb, 128, 0, s>>>(p);
-        else
-            hop_kernel_dirs<SIn, SOut, SX, Lk, Dag, Axpy, kMinCtas, true><<<nsb * p.nrhs, 128, 0, s>>>(p);
+            return launch_dependent(hop_kernel_dirs<SIn, SOut, SX, Lk, Dag, Axpy, kMinCtas, false>, nsb, 128, s, p);
+        return launch_dependent(hop_kernel_dirs<SIn, SOut, SX, Lk, Dag, Axpy, kMinCtas, true>, nsb * p.nrhs, 128, s, p);
     }
-    WEO_CUDA(cudaGetLastError());
-    return WEO_OK;
 }
 
 template <class SIn, class SOut, class SX, class Lk, bool Dag, bool Axpy, int R>

@@ -213,6 +213,7 @@ __device__ __forceinline__ void dirs_block(const HopParams &p, int b, int r, Dir
         for (int k = 0; k < 4; ++k) xv[k] = ld_keep(at(x + 3ll * k * p.vh, (uint32_t)i));
     }
     __syncthreads();
+    pdl_next();
     if (w < 3)
         finish_site<SOut, Dag, Axpy>(p, static_cast<char *>(p.out) + (MULTI ? r * p.out_stride : 0),
                                      sh.chi + 32 * w + lane, w, lane, (uint32_t)i, valid, xv, sh.mx, sh.wd);
@@ -225,6 +226,7 @@ template <class SIn, class SOut, class SX, class Lk, bool Dag, bool Axpy, int MI
 __global__ void __launch_bounds__(128, MINB) hop_kernel_dirs(const HopParams p)
 {
     __shared__ DirsShared<Is16<SOut>::value> sh;
+    pdl_wait();
     const int r = MULTI ? (int)blockIdx.x % p.nrhs : 0;
     int b = MULTI ? (int)blockIdx.x / p.nrhs : (int)blockIdx.x;
     if (p.reverse) b = (MULTI ? (p.vh + 31) / 32 : (int)gridDim.x) - 1 - b;
@@ -299,6 +301,7 @@ template <class Lk, bool Dag, bool Axpy>
 __global__ void __launch_bounds__(128, 3) hop_kernel_pairs(const HopParams p)
 {
     __shared__ double2 part[4 * 12 * 32];
+    pdl_wait();
     const int r = (int)blockIdx.x % p.nrhs;
     int b = (int)blockIdx.x / p.nrhs;
     if (p.reverse) b = (p.vh + 31) / 32 - 1 - b;
@@ -351,6 +354,7 @@ __global__ void __launch_bounds__(128, 4) hop_kernel_rows(const HopParams p)
 {
     constexpr int S0 = Dag ? -1 : 1;
     __shared__ double2 part[4][12 * 16];
+    pdl_wait();
     const int lane = (int)threadIdx.x & 31, w = warp_id();
     const int r = (int)blockIdx.x % p.nrhs;
     int b = (int)blockIdx.x / p.nrhs;
@@ -372,6 +376,7 @@ __global__ void __launch_bounds__(128, 4) hop_kernel_rows(const HopParams p)
     default: pair_rows<3, S0>(p, in, Uf, Ub, nf, nbk, row, o); break;
     }
     __syncthreads();
+    pdl_next();
     // 12 spin-colour components x 16 sites over four warps, the last four over two
     for (int k = 2 * w + row; k < 12; k += 8) {
         double2 xv = make_double2(0.0, 0.0);
