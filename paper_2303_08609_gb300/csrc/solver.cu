@@ -67,6 +67,8 @@ struct SolverState {
     Buffer p64, Ap64;                          // plain FP64 CG
     Buffer xff, eff, tff, oddff;               // float-float true residuals
     cudaStream_t stream = nullptr;
+    cudaStream_t side = nullptr;               // reductions that overlap the operator
+    cudaEvent_t fork = nullptr, join = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // [mixed]
     int graph_chunk[2] = {0, 0};
     int graph_nrhs[2] = {0, 0};
@@ -449,6 +451,9 @@ void solver_destroy(wilson_eo_s *h)
     if (!S) return;
     for (auto &g : S->graph)
         if (g) cudaGraphExecDestroy(g);
+    if (S->fork) cudaEventDestroy(S->fork);
+    if (S->join) cudaEventDestroy(S->join);
+    if (S->side) cudaStreamDestroy(S->side);
     if (S->stream) cudaStreamDestroy(S->stream);
     if (S->host) cudaFreeHost(S->host);
     Buffer *bufs[] = {&S->scal, &S->x64, &S->b64, &S->r64, &S->e64, &S->t64, &S->odd64,
@@ -466,6 +471,9 @@ static int solver_state(wilson_eo_s *h, SolverState **out)
         h->solver = S;
         cudaError_t e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
         if (e != cudaSuccess) return fail_cuda(e, "cudaStreamCreateWithFlags", __FILE__, __LINE__);
+        WEO_CUDA(cudaStreamCreateWithFlags(&S->side, cudaStreamNonBlocking));
+        WEO_CUDA(cudaEventCreateWithFlags(&S->fork, cudaEventDisableTiming));
+        WEO_CUDA(cudaEventCreateWithFlags(&S->join, cudaEventDisableTiming));
         e = cudaMallocHost(&S->host, sizeof(SolveScalars) * kMaxRhs);
         if (e != cudaSuccess) return fail_cuda(e, "cudaMallocHost", __FILE__, __LINE__);
         WEO_TRY(S->scal.ensure(sizeof(SolveScalars) * kMaxRhs));
@@ -539,28 +547,34 @@ static int normal_op(wilson_eo_s *h, SolverState *S, const PackedGauge &g, Buffe
     return meo_with(h, g, odd, out, e, S->nrhs, true, s);
 }
 
-// One CG iteration of every right-hand side. mixed: low-precision vectors
-// (float2) with operator g; otherwise FP64 vectors.
-static int cg_iteration(wilson_eo_s *h, SolverState *S, const PackedGauge &g, bool mixed,
-                        cudaStream_t s)
+// One CG iteration of every right-hand side on vectors of T2 (float2: the
+// low-precision operator g, double2: FP64). The step length needs only M p, so its
+// norm runs on the side stream beside the two hops of M^dag.
+template <typename T2>
+static int cg_step(wilson_eo_s *h, SolverState *S, const PackedGauge &g, Buffer &odd, void *x, void *r, void *p,
+                   void *mp, void *ap, cudaStream_t s)
 {
     const long long n = 12 * h->vh;
     const dim3 grid(red_grid(n), S->nrhs);
     SolveScalars *sc = dev_scal(S);
-    if (mixed) {
-        WEO_TRY(normal_op(h, S, g, S->oddlo, S->t32.ptr, S->Ap.ptr, S->p.ptr, s));
-        WEO_TRY(launch_dependent(k_norm2<float2>, grid, kRedThreads, s, (const float2 *)S->t32.ptr, n, sc, 2));
-        WEO_TRY(launch_dependent(k_cg_update<float2>, grid, kRedThreads, s, (float2 *)S->rs.ptr,
-                                 (const float2 *)S->Ap.ptr, n, sc));
-        return launch_dependent(k_cg_dir<float2>, grid, kRedThreads, s, (float2 *)S->xs.ptr, (float2 *)S->p.ptr,
-                                (const float2 *)S->rs.ptr, n, sc);
-    }
-    WEO_TRY(normal_op(h, S, g, S->odd64, S->e64.ptr, S->Ap64.ptr, S->p64.ptr, s));
-    WEO_TRY(launch_dependent(k_norm2<double2>, grid, kRedThreads, s, (const double2 *)S->e64.ptr, n, sc, 2));
-    WEO_TRY(launch_dependent(k_cg_update<double2>, grid, kRedThreads, s, (double2 *)S->r64.ptr,
-                             (const double2 *)S->Ap64.ptr, n, sc));
-    return launch_dependent(k_cg_dir<double2>, grid, kRedThreads, s, (double2 *)S->x64.ptr, (double2 *)S->p64.ptr,
-                            (const double2 *)S->r64.ptr, n, sc);
+    WEO_TRY(meo_with(h, g, odd, mp, p, S->nrhs, false, s));
+    WEO_CUDA(cudaEventRecord(S->fork, s));
+    WEO_CUDA(cudaStreamWaitEvent(S->side, S->fork, 0));
+    k_norm2<T2><<<grid, kRedThreads, 0, S->side>>>((const T2 *)mp, n, sc, 2);
+    WEO_CUDA(cudaGetLastError());
+    WEO_CUDA(cudaEventRecord(S->join, S->side));
+    WEO_TRY(meo_with(h, g, odd, ap, mp, S->nrhs, true, s));
+    WEO_CUDA(cudaStreamWaitEvent(s, S->join, 0));
+    k_cg_update<T2><<<grid, kRedThreads, 0, s>>>((T2 *)r, (const T2 *)ap, n, sc);
+    WEO_CUDA(cudaGetLastError());
+    return launch_dependent(k_cg_dir<T2>, grid, kRedThreads, s, (T2 *)x, (T2 *)p, (const T2 *)r, n, (const SolveScalars *)sc);
+}
+
+static int cg_iteration(wilson_eo_s *h, SolverState *S, const PackedGauge &g, bool mixed,
+                        cudaStream_t s)
+{
+    return mixed ? cg_step<float2>(h, S, g, S->oddlo, S->xs.ptr, S->rs.ptr, S->p.ptr, S->t32.ptr, S->Ap.ptr, s)
+                 : cg_step<double2>(h, S, g, S->odd64, S->x64.ptr, S->r64.ptr, S->p64.ptr, S->e64.ptr, S->Ap64.ptr, s);
 }
 
 // Run `k` iterations, from a captured graph when enabled.
