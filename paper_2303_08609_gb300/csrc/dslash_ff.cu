@@ -8,11 +8,12 @@
 // which was bound by their issue (70 %). As in weo_split.cuh a CTA of 128 threads
 // takes 32 output sites and warp mu the directions +-mu; three warps add the four
 // pairs, and the second hop writes complex128 itself. us per M_eo on complex128
-// spinors, one site per thread -> here: 8^4 41.9 -> 17.1, 16^3 x 32 119 -> 73.8,
-// 24^3 x 48 430 -> 349, 32^3 x 64 1304 -> 1059; relative error 2.4e-15 -> 2.3e-15.
-// Of the 349, 38 are the conversion of the input and 311 the two hops: issue 43 % of
-// cycles, bound by the latency of the loads at 16 warps per SM (128 registers; three
-// CTAs per SM without the cap 386, five or six with spills 429 and 407).
+// spinors, one site per thread -> here: 8^4 41.9 -> 14.3, 16^3 x 32 119 -> 67.2,
+// 24^3 x 48 430 -> 299, 32^3 x 64 1304 -> 915; relative error 2.4e-15 -> 2.3e-15.
+// Of the 299, 38 are the conversion of the input and 261 the two hops: issue 45-50 %
+// of cycles, bound by the latency of the loads at 16 warps per SM (117 registers;
+// three CTAs per SM 301, five or six with spills 314 and 329). Loading both links
+// again for each spin row was 344; fetching the next row's values ahead 313.
 #include "weo_internal.h"
 #include "weo_split.cuh"
 
@@ -148,7 +149,8 @@ __device__ __forceinline__ void ff_row(const FCRows &r, float sg, const FFLink &
 }
 
 // Both hops of direction mu for one site: P + Q (three colours of spin rows 0, 1)
-// and P - Q, left in `out`. One copy of this code serves two of the directions and
+// and P - Q, left in `out` (P waits there for Q, so each link is loaded once for
+// both rows). One copy of this code serves two of the directions and
 // both spin rows: unrolled over all of them the kernel is 6000 instructions, and
 // warps waited for instructions 40 % of the time.
 template <bool ROT>
@@ -157,22 +159,29 @@ __device__ __forceinline__ void ff_pair(const HopParams &p, const float2 *in, in
 {
     const char *gf = p.gauge + (2 * mu + p.out_parity) * p.gauge_pb;
     const char *gb = p.gauge + (2 * mu + (p.out_parity ^ 1)) * p.gauge_pb;
+    // project<MU, S>: the sign of x, y, z, t for spin row s, and the partner's spin
+    auto sign = [&](int s) { return mu == 3 || ((mu == 1 || mu == 2) && s) ? -s0 : s0; };
+    auto row = [&](int s) { return in + 3ll * s * p.vh; };
+    auto partner = [&](int s) { return in + 3ll * (mu < 2 ? 3 - s : 2 + s) * p.vh; };
+    FFLink U;
+    load_ff_link(gf, p.vh, i, U);
 #pragma unroll 1
     for (int s = 0; s < 2; ++s) {
-        // project<MU, S>: the sign of x, y, z, t for spin row s, and the partner's spin
-        const float sg = (mu == 3 || ((mu == 1 || mu == 2) && s)) ? -s0 : s0;
-        const float2 *a = in + 3ll * s * p.vh, *b = in + 3ll * (mu < 2 ? 3 - s : 2 + s) * p.vh;
-        FC P[3], Q[3];
-        const FCRows rf = load_rows(a, b, p.vh, nf);
-        FFLink U, V;
-        load_ff_link(gf, p.vh, i, U);
-        const FCRows rb = load_rows(a, b, p.vh, nb);
-        load_ff_link(gb, p.vh, nb, V);
-        ff_row<ROT, true>(rf, sg, U, P);
-        ff_row<ROT, false>(rb, -sg, V, Q);
+        FC P[3];
+        ff_row<ROT, true>(load_rows(row(s), partner(s), p.vh, nf), sign(s), U, P);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) out[32 * (3 * s + k)] = make_float4(P[k].h.x, P[k].h.y, P[k].l.x, P[k].l.y);
+    }
+    load_ff_link(gb, p.vh, nb, U);
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {
+        FC Q[3];
+        ff_row<ROT, false>(load_rows(row(s), partner(s), p.vh, nb), -sign(s), U, Q);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const FC u = add_pair(P[k], Q[k], f2(1.f)), d = add_pair(P[k], Q[k], f2(-1.f));
+            const float4 f = out[32 * (3 * s + k)];
+            const FC P = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+            const FC u = add_pair(P, Q[k], f2(1.f)), d = add_pair(P, Q[k], f2(-1.f));
             out[32 * (3 * s + k)] = make_float4(u.h.x, u.h.y, u.l.x, u.l.y);
             out[32 * (6 + 3 * s + k)] = make_float4(d.h.x, d.h.y, d.l.x, d.l.y);
         }
