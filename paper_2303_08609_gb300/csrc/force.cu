@@ -76,17 +76,15 @@ __device__ __forceinline__ void outer_acc(cx<T> G[3][3], const cx<T> hp[2][3], c
 
 // The result for link (mu, x) from the sum of its two outer products: the gradient
 // G, or the force TA(G U^dag), as 18 reals in m.
-template <class Lk, int MU, typename T>
-__device__ __forceinline__ void grad_finish(const GradParams &p, int par, long long i, cx<T> G[3][3], T m[18])
+template <typename T>
+__device__ __forceinline__ void grad_finish(const GradParams &p, bool force, const cx<T> U[3][3], cx<T> G[3][3], T m[18])
 {
     const T sc = T(p.scale);
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int b = 0; b < 3; ++b) G[a][b] = cscale(G[a][b], sc);
-    if (p.force) {
-        cx<T> U[3][3];
-        Lk::load(p.gauge + (2 * MU + par) * p.gauge_pb, p.vh, i, U);
+    if (force) {
         cx<T> W[3][3];  // G U^dag
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -120,7 +118,7 @@ __device__ __forceinline__ void grad_finish(const GradParams &p, int par, long l
 // own0, own1: the site's own fields (g, phi on even sites; t, w on odd sites).
 // even x: G = (1-g)g(x) (x) (1-g)t(x+mu) + (1+g)phi(x) (x) (1+g)w(x+mu);
 // odd x:  G = (1+g)t(x) (x) (1+g)g(x+mu) + (1-g)w(x) (x) (1-g)phi(x+mu)
-template <class Sp, class Lk, int MU>
+template <class Sp, class Lk, bool FORCE, int MU>
 __device__ __forceinline__ void grad_link(const GradParams &p, int par, long long i, long long nb,
                                           const cx<typename Sp::real> own0[12],
                                           const cx<typename Sp::real> own1[12],
@@ -128,7 +126,8 @@ __device__ __forceinline__ void grad_link(const GradParams &p, int par, long lon
 {
     using T = typename Sp::real;
     const T S1 = par ? T(-1) : T(1);
-    cx<T> n0[12], n1[12], ha[2][3], hb[2][3];
+    cx<T> n0[12], n1[12], ha[2][3], hb[2][3], U[3][3];
+    if (FORCE) Lk::load(p.gauge + (2 * MU + par) * p.gauge_pb, p.vh, i, U);
     Sp::load(par ? p.g : p.t, p.vh, nb, n0);
     Sp::load(par ? p.phi : p.w, p.vh, nb, n1);
     cx<T> G[3][3];
@@ -142,7 +141,7 @@ __device__ __forceinline__ void grad_link(const GradParams &p, int par, long lon
     proj_rt<MU>(own1, -S1, ha);
     proj_rt<MU>(n1, -S1, hb);
     outer_acc(G, ha, hb);
-    grad_finish<Lk, MU>(p, par, i, G, m);
+    grad_finish(p, FORCE, U, G, m);
 }
 
 // Stage the block's matrices for one direction in shared memory and write them
@@ -172,9 +171,13 @@ __device__ __forceinline__ void write_links(const GradParams &p, int mu, long lo
 
 // FP32: one thread per lattice site (lexicographic, both parities): it computes the
 // four links based there; each block writes its links per direction as one
-// contiguous range.
-template <class Sp, class Lk>
-__global__ void __launch_bounds__(kGradThreads) link_grad_kernel(const GradParams p)
+// contiguous range. Bound by the latency of the loads: 16 warps per SM (128 registers;
+// three CTAs per SM 113 us, five with spills 90 for the gradient) keep HBM at 54 % and
+// issue at 35 % of cycles. So the force's own link is fetched together with the
+// neighbours, not after the products: 112.8 -> 107.2 us at 24^3 x 48, 27.0 -> 25.3 at
+// 16^3 x 32 (the gradient alone 78.5).
+template <class Sp, class Lk, bool FORCE>
+__global__ void __launch_bounds__(kGradThreads, 4) link_grad_kernel(const GradParams p)
 {
     using T = typename Sp::real;
     __shared__ __align__(16) T sh[18 * kGradThreads];
@@ -203,13 +206,13 @@ __global__ void __launch_bounds__(kGradThreads) link_grad_kernel(const GradParam
     Sp::load(par ? p.t : p.g, p.vh, i, own0);
     Sp::load(par ? p.w : p.phi, p.vh, i, own1);
     T m[18];
-    grad_link<Sp, Lk, 0>(p, par, i, n_x, own0, own1, m);
+    grad_link<Sp, Lk, FORCE, 0>(p, par, i, n_x, own0, own1, m);
     write_links(p, 0, lex0, nvalid, m, sh);
-    grad_link<Sp, Lk, 1>(p, par, i, n_y, own0, own1, m);
+    grad_link<Sp, Lk, FORCE, 1>(p, par, i, n_y, own0, own1, m);
     write_links(p, 1, lex0, nvalid, m, sh);
-    grad_link<Sp, Lk, 2>(p, par, i, n_z, own0, own1, m);
+    grad_link<Sp, Lk, FORCE, 2>(p, par, i, n_z, own0, own1, m);
     write_links(p, 2, lex0, nvalid, m, sh);
-    grad_link<Sp, Lk, 3>(p, par, i, n_t, own0, own1, m);
+    grad_link<Sp, Lk, FORCE, 3>(p, par, i, n_t, own0, own1, m);
     write_links(p, 3, lex0, nvalid, m, sh);
 }
 
@@ -233,16 +236,18 @@ __device__ __forceinline__ void grad_link_f64(const GradParams &p, int par, uint
     };
     term(par ? p.t : p.g, par ? p.g : p.t, S1);
     term(par ? p.w : p.phi, par ? p.phi : p.w, -S1);
-    grad_finish<Lk, MU>(p, par, i, G, m);
+    cx<double> U[3][3];
+    if (p.force) Lk::load(p.gauge + (2 * MU + par) * p.gauge_pb, p.vh, i, U);
+    grad_finish(p, p.force != 0, U, G, m);
 }
 
 // FP64: a CTA takes 32 consecutive sites, warp mu of it the 32 links of direction mu
 // based there, which it stages in shared memory and writes as one contiguous range.
 // Bound by the FP64 pipe; against one thread per site (236 registers, CTAs of 128
 // sites) the work spreads evenly over the SMs: force 56.5 -> 18.6 us at 8^4, 343 ->
-// 328 at 16^3 x 32, 1675 -> 1640 at 24^3 x 48. In FP32, where the site's own fields
+// 326 at 16^3 x 32, 1675 -> 1648 at 24^3 x 48. In FP32, where the site's own fields
 // read by four warps cost more than the shorter chains gain, it measured 123 against
-// 114 us at 24^3 x 48.
+// 113 us at 24^3 x 48.
 template <class Lk>
 __global__ void __launch_bounds__(4 * kGradSites, 3) link_grad_kernel_f64(const GradParams p)
 {
@@ -289,7 +294,10 @@ template <class Lk>
 static int launch_grad_f32(const GradParams &p, cudaStream_t s)
 {
     const unsigned blocks = (unsigned)((2LL * p.vh + kGradThreads - 1) / kGradThreads);
-    link_grad_kernel<SpF32, Lk><<<blocks, kGradThreads, 0, s>>>(p);
+    if (p.force)
+        link_grad_kernel<SpF32, Lk, true><<<blocks, kGradThreads, 0, s>>>(p);
+    else
+        link_grad_kernel<SpF32, Lk, false><<<blocks, kGradThreads, 0, s>>>(p);
     WEO_CUDA(cudaGetLastError());
     return WEO_OK;
 }
