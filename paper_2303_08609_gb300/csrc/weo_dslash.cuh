@@ -83,23 +83,23 @@ struct HopParams {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// h = psi_up - S A_mu psi_dn for one colour
-template <int MU, int S, typename R>
+// h = psi_up - S A_mu psi_dn for one colour, times the factor n of a 16-bit load
+template <int MU, int S, typename R, class N = NoScale>
 __device__ __forceinline__ void project(const cx<R> p0, const cx<R> p1, const cx<R> p2,
-                                        const cx<R> p3, cx<R> &h0, cx<R> &h1)
+                                        const cx<R> p3, cx<R> &h0, cx<R> &h1, N n = N())
 {
     if (MU == 0) {  // A = -i sigma_1: A psi_dn = (-i p3, -i p2)
-        h0 = S > 0 ? cadd(p0, cmuli(p3)) : csub(p0, cmuli(p3));
-        h1 = S > 0 ? cadd(p1, cmuli(p2)) : csub(p1, cmuli(p2));
+        h0 = S > 0 ? cadd(p0, cmuli(p3), n) : csub(p0, cmuli(p3), n);
+        h1 = S > 0 ? cadd(p1, cmuli(p2), n) : csub(p1, cmuli(p2), n);
     } else if (MU == 1) {  // A = -i sigma_2 = [[0,-1],[1,0]]: A psi_dn = (-p3, p2)
-        h0 = S > 0 ? cadd(p0, p3) : csub(p0, p3);
-        h1 = S > 0 ? csub(p1, p2) : cadd(p1, p2);
+        h0 = S > 0 ? cadd(p0, p3, n) : csub(p0, p3, n);
+        h1 = S > 0 ? csub(p1, p2, n) : cadd(p1, p2, n);
     } else if (MU == 2) {  // A = -i sigma_3: A psi_dn = (-i p2, i p3)
-        h0 = S > 0 ? cadd(p0, cmuli(p2)) : csub(p0, cmuli(p2));
-        h1 = S > 0 ? csub(p1, cmuli(p3)) : cadd(p1, cmuli(p3));
+        h0 = S > 0 ? cadd(p0, cmuli(p2), n) : csub(p0, cmuli(p2), n);
+        h1 = S > 0 ? csub(p1, cmuli(p3), n) : cadd(p1, cmuli(p3), n);
     } else {  // A = 1
-        h0 = S > 0 ? csub(p0, p2) : cadd(p0, p2);
-        h1 = S > 0 ? csub(p1, p3) : cadd(p1, p3);
+        h0 = S > 0 ? csub(p0, p2, n) : cadd(p0, p2, n);
+        h1 = S > 0 ? csub(p1, p3, n) : cadd(p1, p3, n);
     }
 }
 
@@ -157,8 +157,7 @@ __device__ __forceinline__ void hop_dir(cx<T> (&acc)[R][12], const HopParams &p,
         // spin-colour index k = 3*spin + colour
         cx<T> h[2][3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c]);
-        scale_rows(h, n);
+        for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c], n);
         cx<T> w[2][3];
         link_mul<FWD>(U, h, w);
 #pragma unroll
@@ -428,8 +427,7 @@ __device__ __forceinline__ void hop_dir_shared(cx<float> (&acc)[RP][12], const H
         const auto n = SIn::load(static_cast<const char *>(p.in) + (rhs + r * step) * p.in_stride, p.vh, nb, v);
         cx<float> h[2][3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c]);
-        scale_rows(h, n);
+        for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c], n);
         cx<float> w[2][3];
 #pragma unroll
         for (int sp = 0; sp < 2; ++sp)

@@ -148,18 +148,26 @@ __device__ __forceinline__ const T *at(const T *plane, I i)
 
 // ---------------------------------------------------------------- spinors --
 // load() returns the factor that the values still need: none, or the site's norm
-// of the 16-bit formats. The hops apply it to the projected spinor (scale_rows),
-// 12 values instead of 24, with a multiplication that cannot be contracted into
-// the projection's additions, so every kernel rounds alike.
+// of the 16-bit formats, which the projection applies (project in weo_dslash.cuh).
 struct NoScale {};
 
+// (a + b) n and (a - b) n. With a norm n the value b n is rounded first and a n
+// added to it in one fused operation, spelled out so that every kernel rounds
+// alike: where a result is rounded to 16 bits again, another order of these
+// operations moves single elements by a whole step of the format, 2^-8 of the
+// site's norm with BF16. The 24 operations per direction are as many as the
+// projection and a multiplication of its 12 results would take.
 template <typename R>
-__device__ __forceinline__ void scale_rows(cx<R> (&)[2][3], NoScale) {}
-__device__ __forceinline__ void scale_rows(cx<float> (&h)[2][3], float n)
+__device__ __forceinline__ cx<R> cadd(cx<R> a, cx<R> b, NoScale) { return cadd(a, b); }
+template <typename R>
+__device__ __forceinline__ cx<R> csub(cx<R> a, cx<R> b, NoScale) { return csub(a, b); }
+__device__ __forceinline__ cx<float> cadd(cx<float> a, cx<float> b, float n)
 {
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-        h[k / 3][k % 3] = {__fmul_rn(h[k / 3][k % 3].r, n), __fmul_rn(h[k / 3][k % 3].i, n)};
+    return {fmaf(a.r, n, __fmul_rn(b.r, n)), fmaf(a.i, n, __fmul_rn(b.i, n))};
+}
+__device__ __forceinline__ cx<float> csub(cx<float> a, cx<float> b, float n)
+{
+    return {fmaf(a.r, n, -__fmul_rn(b.r, n)), fmaf(a.i, n, -__fmul_rn(b.i, n))};
 }
 
 struct SpF64 {
@@ -290,15 +298,18 @@ using SpB16 = Sp16<B16Traits>;
 
 // ------------------------------------------------------------------ links --
 
-// conj(a b - c d) in eight operations, none of which the compiler may contract
-// in another way (every kernel rounds alike)
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-template <typename R>
-__device__ __forceinline__ cx<R> cross_conj(cx<R> a, cx<R> b, cx<R> c, cx<R> d)
+// conj(a b - c d) in eight operations, for the FP64 pipe
+__device__ __forceinline__ cx<double> cross_conj(cx<double> a, cx<double> b, cx<double> c, cx<double> d)
 {
-    return {fma(c.i, d.i, fma(-c.r, d.r, fma(-a.i, b.i, mul_rn(a.r, b.r)))),
-            fma(c.i, d.r, fma(c.r, d.i, fma(-a.i, b.r, mul_rn(-a.r, b.i))))};
+    return {fma(c.i, d.i, fma(-c.r, d.r, fma(-a.i, b.i, __dmul_rn(a.r, b.r)))),
+            fma(c.i, d.r, fma(c.r, d.i, fma(-a.i, b.r, __dmul_rn(-a.r, b.i))))};
+}
+// FP32, also under 16-bit storage: the two products rounded apart, then subtracted.
+// The eight operations of the FP64 form round otherwise, which 16-bit results
+// multiply (see cadd with a norm above).
+__device__ __forceinline__ cx<float> cross_conj(cx<float> a, cx<float> b, cx<float> c, cx<float> d)
+{
+    return cconj(csub(cmul(a, b), cmul(c, d)));
 }
 
 template <typename R>

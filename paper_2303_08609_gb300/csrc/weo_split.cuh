@@ -42,8 +42,7 @@ __device__ __forceinline__ void dir_chi(const cx<float> U[3][3], const cx<float>
     constexpr int S = FWD ? S0 : -S0;
     cx<float> h[2][3], w[2][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c]);
-    scale_rows(h, scale);
+    for (int c = 0; c < 3; ++c) project<MU, S>(v[c], v[3 + c], v[6 + c], v[9 + c], h[0][c], h[1][c], scale);
     link_mul<FWD>(U, h, w);
 #pragma unroll
     for (int k = 0; k < 6; ++k) out[32 * k] = make_float2(w[k / 3][k % 3].r, w[k / 3][k % 3].i);
