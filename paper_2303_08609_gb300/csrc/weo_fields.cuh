@@ -111,12 +111,16 @@ template <typename T>
 __device__ __forceinline__ cx<T> cscale(cx<T> a, T s) { return {a.r * s, a.i * s}; }
 
 // ------------------------------------------------------------ loads/stores --
-// Spinor neighbour reads are re-used by up to eight output sites: plain cached
-// loads. Links are used once per pass: streaming loads (evict-first) so they do
-// not push the spinor working set out of L2.
+// Spinor neighbour reads are re-used by up to eight output sites: loads cached in
+// L1 and L2. Not the read-only path (__ldg): it is for memory that nobody writes
+// while the kernel runs, and a hop launched as a programmatic dependent is resident
+// while its predecessor still writes the spinor that it reads after pdl_wait; the
+// batch's second hop reads what its first hop wrote in the same launch. Links are
+// used once per pass: streaming loads (evict-first) so they do not push the spinor
+// working set out of L2.
 
 template <typename T>
-__device__ __forceinline__ T ld_keep(const T *p) { return __ldg(p); }
+__device__ __forceinline__ T ld_keep(const T *p) { return __ldca(p); }
 template <typename T>
 __device__ __forceinline__ T ld_stream(const T *p) { return __ldcs(p); }
 
