@@ -172,8 +172,7 @@ int wilson_eo_force(wilson_eo_t h, void *force, void *dS_dphi_e, const void *phi
  *              vectors, with reliable updates: whenever the iterated residual
  *              has fallen by `delta` (default 0.1) the FP32 increment is added
  *              to the FP64 solution and the residual is recomputed as b - A x
- *              with the FP64 operator. Reductions accumulate in FP64 (over FP32
- *              vectors in float-float, 48 bits).
+ *              with the FP64 operator. Reductions accumulate in FP64.
  * Convergence: |b - A x| / |b| <= tol with the residual recomputed in FP64 from
  * the returned x (true_relres_out). Returns WEO_OK, WEO_ERR_NOT_CONVERGED
  * (maxiter iterations done, or -- mixed mode -- the true residual grew 10^4-fold

@@ -51,6 +51,7 @@ struct SolveScalars {
     double alpha;
     double beta;
     double red;      // result of the last plain reduction
+    double scale[2]; // the low-precision vectors hold the system's ones divided by this power of two; its inverse
     int nonfinite;   // set when a reduction or a scalar is NaN / Inf or pAp <= 0
     int active;      // 0 once this right-hand side has converged
     unsigned int counter;
@@ -137,56 +138,44 @@ __device__ __forceinline__ double re_dot(T2 a, T2 b) { return double(a.x) * b.x 
 
 // FP32 vectors are read as float4 (two complex numbers; n = 12 V/2 is even and
 // every right-hand side starts on a 16-byte boundary). The squares of the four
-// float4 that a thread has in flight are summed in FP32, and those group sums are
-// accumulated, over the thread, the warp and the block, as a float-float number
-// (error-free sums, 48 bits, far below the rounding of the FP32 squares): each FP64
-// instruction of a warp takes 16 cycles of the SM's FP64 pipe. At 16^3 x 32 the
-// norm of M p took 8.5 us with FP64 sums and takes 6.0, the residual update 9.1
-// and 8.3.
+// float4 that a thread has in flight are summed in FP32 and those group sums (of
+// the float4 themselves at the end of the vector) accumulated in FP64, whose range
+// the sums need: vectors of 1e17 an element have |a|^2 beyond FP32's. Each FP64
+// instruction of a warp takes 16 cycles of the SM's FP64 pipe, so per-element FP64
+// arithmetic would bound these kernels.
 __device__ __forceinline__ float sq4(float4 q) { return q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w; }
-
-struct Sum2 {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float x, float xl = 0.f)
-    {
-        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-        const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b));
-        h = s;
-        l = __fadd_rn(l, __fadd_rn(e, xl));
-    }
-};
-
-// sum over the block, valid in thread 0
-__device__ __forceinline__ double block_sum(Sum2 v)
-{
-    __shared__ float2 sh[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h = __shfl_down_sync(0xffffffffu, v.h, o), l = __shfl_down_sync(0xffffffffu, v.l, o);
-        v.add(h, l);
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[w] = make_float2(v.h, v.l);
-    __syncthreads();
-    if (threadIdx.x != 0) return 0.0;
-    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) v.add(sh[k].x, sh[k].y);
-    return double(v.h) + double(v.l);
-}
 
 __device__ __forceinline__ long long grid_stride() { return (long long)gridDim.x * blockDim.x; }
 __device__ __forceinline__ long long grid_index() { return blockIdx.x * (long long)blockDim.x + threadIdx.x; }
 
-// sum of |a_k|^2 over n complex values, this thread's share
-__device__ __forceinline__ Sum2 sum_sq(const float2 *a, long long n)
+// the squares of four float4, of which the first `in` are there (at least one)
+__device__ __forceinline__ double sum_sq4(const float4 q[4], int in)
 {
-    Sum2 v;
-    const float4 *a4 = reinterpret_cast<const float4 *>(a), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (in == 4) return double((sq4(q[0]) + sq4(q[1])) + (sq4(q[2]) + sq4(q[3])));
+    double v = double(sq4(q[0]));
+#pragma unroll
+    for (int j = 1; j < 3; ++j)
+        if (j < in) v += double(sq4(q[j]));
+    return v;
+}
+// how many of k, k + st, k + 2 st, k + 3 st lie below n (k does)
+__device__ __forceinline__ int in_flight(long long k, long long st, long long n)
+{
+    return 1 + (k + st < n) + (k + 2 * st < n) + (k + 3 * st < n);
+}
+
+// sum of |a_k|^2 over n complex values, this thread's share
+__device__ __forceinline__ double sum_sq(const float2 *a, long long n)
+{
+    double v = 0.0;
+    const float4 *a4 = reinterpret_cast<const float4 *>(a);
     const long long n4 = n >> 1, st = grid_stride();
     for (long long k = grid_index(); k < n4; k += 4 * st) {
-        const float4 q0 = a4[k], q1 = k + st < n4 ? a4[k + st] : zero, q2 = k + 2 * st < n4 ? a4[k + 2 * st] : zero,
-                     q3 = k + 3 * st < n4 ? a4[k + 3 * st] : zero;
-        v.add((sq4(q0) + sq4(q1)) + (sq4(q2) + sq4(q3)));
+        const int in = in_flight(k, st, n4);
+        float4 q[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[j] = a4[j < in ? k + j * st : k];
+        v += sum_sq4(q, in);
     }
     return v;
 }
@@ -210,9 +199,9 @@ __global__ void __launch_bounds__(kRedThreads) k_norm2(const T2 *a, long long n,
     SolveScalars *sc = scs + blockIdx.y;
     if (mode >= 1 && !sc->active) return;
     if (mode == 2 && sc->nonfinite) return;
-    const auto part = sum_sq(a + blockIdx.y * n, n);
+    double v = sum_sq(a + blockIdx.y * n, n);
     pdl_next();
-    double v = block_sum(part);
+    v = block_sum(v);
     double tot;
     if (finish_reduction(sc, v, &tot) && threadIdx.x == 0) {
         if (mode == 0) {
@@ -256,24 +245,23 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(T2 *r, const T2 *Ap, 
         float4 *r4 = reinterpret_cast<float4 *>(r);
         const float4 *a4 = reinterpret_cast<const float4 *>(Ap);
         const long long n4 = n >> 1, st = grid_stride();
-        Sum2 q;
         for (long long k0 = grid_index(); k0 < n4; k0 += 4 * st) {
+            const int in = in_flight(k0, st, n4);
             float4 rv[4], av[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const bool in = k0 + j * st < n4;
-                rv[j] = in ? r4[k0 + j * st] : make_float4(0.f, 0.f, 0.f, 0.f);
-                av[j] = in ? a4[k0 + j * st] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const long long k = j < in ? k0 + j * st : k0;
+                rv[j] = r4[k];
+                av[j] = a4[k];
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 axpy4(rv[j], -alpha, av[j]);
-                if (k0 + j * st < n4) r4[k0 + j * st] = rv[j];
+                if (j < in) r4[k0 + j * st] = rv[j];
             }
-            q.add((sq4(rv[0]) + sq4(rv[1])) + (sq4(rv[2]) + sq4(rv[3])));
+            v += sum_sq4(rv, in);
         }
         pdl_next();
-        v = block_sum(q);
     } else {
         FOR_ELEMENTS(k) {
             T2 rv = r[k];
@@ -283,8 +271,8 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(T2 *r, const T2 *Ap, 
             r[k] = rv;
             v += re_dot(rv, rv);
         }
-        v = block_sum(v);
     }
+    v = block_sum(v);
     double tot;
     if (finish_reduction(sc, v, &tot) && threadIdx.x == 0) {
         if (!isfinite(tot) || !isfinite(tot / sc->rr)) {
@@ -405,27 +393,29 @@ __global__ void __launch_bounds__(kRedThreads) k_residual_ff(double2 *r, const d
     if (finish_reduction(sc, v, &tot) && threadIdx.x == 0) sc->red = tot;
 }
 
-// d = s over all right-hand sides (n_total elements)
-template <typename D2, typename S2>
-__global__ void k_convert(D2 *d, const S2 *s, long long n)
+// d = s / scale, for each right-hand side (blockIdx.y)
+__global__ void k_convert(float2 *d, const double2 *s, long long n, const SolveScalars *scs)
 {
+    const double f = scs[blockIdx.y].scale[1];
+    d += blockIdx.y * n;
+    s += blockIdx.y * n;
     FOR_ELEMENTS(k) {
-        const S2 v = s[k];
-        D2 o;
-        o.x = v.x;
-        o.y = v.y;
-        d[k] = o;
+        const double2 v = s[k];
+        d[k] = make_float2((float)(v.x * f), (float)(v.y * f));
     }
 }
 
-// x64 += xs ; xs = 0 (n_total elements)
-__global__ void k_accumulate(double2 *x, float2 *xs, long long n)
+// x64 += scale xs ; xs = 0, for each right-hand side
+__global__ void k_accumulate(double2 *x, float2 *xs, long long n, const SolveScalars *scs)
 {
+    const double f = scs[blockIdx.y].scale[0];
+    x += blockIdx.y * n;
+    xs += blockIdx.y * n;
     FOR_ELEMENTS(k) {
         const float2 v = xs[k];
         double2 a = x[k];
-        a.x += v.x;
-        a.y += v.y;
+        a.x = fma(f, double(v.x), a.x);
+        a.y = fma(f, double(v.y), a.y);
         x[k] = a;
         xs[k] = make_float2(0.f, 0.f);
     }
@@ -795,8 +785,18 @@ static int solve_impl(wilson_eo_s *h, double tol, int maxiter, int mixed, int *i
         WEO_TRY(S->p.ensure(b32));
         WEO_TRY(S->Ap.ensure(b32));
         WEO_TRY(S->t32.ensure(b32));
+        // the inner system is that of r / scale, |r / scale| in [1, 2) at the start: its
+        // residuals' squares stay inside FP32's range whatever that of b is, and a power
+        // of two changes no rounding
+        std::vector<double> scale(R, 1.0);
+        for (int r = 0; r < R; ++r) {
+            if (rr_true[r] > 0.0) scale[r] = ldexp(1.0, std::max(-1000, std::min(1000, ilogb(sqrt(rr_true[r])))));
+            const double both[2] = {scale[r], 1.0 / scale[r]};
+            WEO_CUDA(cudaMemcpyAsync(static_cast<char *>(S->scal.ptr) + r * sizeof(SolveScalars) + offsetof(SolveScalars, scale),
+                                     both, sizeof both, cudaMemcpyHostToDevice, s));
+        }
         WEO_CUDA(cudaMemsetAsync(S->xs.ptr, 0, b32, s));
-        k_convert<float2, double2><<<flat_grid(nt), 256, 0, s>>>((float2 *)S->rs.ptr, (const double2 *)S->r64.ptr, nt);
+        k_convert<<<dim3(flat_grid(n), R), 256, 0, s>>>((float2 *)S->rs.ptr, (const double2 *)S->r64.ptr, n, sc);
         WEO_CUDA(cudaMemcpyAsync(S->p.ptr, S->rs.ptr, b32, cudaMemcpyDeviceToDevice, s));
         k_norm2<float2><<<grid, kRedThreads, 0, s>>>((const float2 *)S->rs.ptr, n, sc, 1);
         WEO_CUDA(cudaGetLastError());
@@ -820,7 +820,7 @@ static int solve_impl(wilson_eo_s *h, double tol, int maxiter, int mixed, int *i
                     restart[r] = 1;
                     update = true;
                 }
-                const double rr = S->host[r].rr;
+                const double rr = S->host[r].rr * scale[r] * scale[r];
                 if (sqrt(rr) < S->delta * r_max[r] || rr <= target[r]) update = true;
                 // an iterated residual far above the last true one: check the
                 // true residual now rather than after the iteration has run away
@@ -829,7 +829,7 @@ static int solve_impl(wilson_eo_s *h, double tol, int maxiter, int mixed, int *i
             if (!update) continue;
             // reliable update of every system: fold the increments into x and
             // recompute the residuals in FP64
-            k_accumulate<<<flat_grid(nt), 256, 0, s>>>((double2 *)S->x64.ptr, (float2 *)S->xs.ptr, nt);
+            k_accumulate<<<dim3(flat_grid(n), R), 256, 0, s>>>((double2 *)S->x64.ptr, (float2 *)S->xs.ptr, n, sc);
             WEO_CUDA(cudaGetLastError());
             WEO_TRY(update_residual(h, S, *ghi, ff, active, target));
             S->reliable_updates += 1;
@@ -855,7 +855,7 @@ static int solve_impl(wilson_eo_s *h, double tol, int maxiter, int mixed, int *i
                                  "grew 1e4-fold); its operator is too far from the FP64 one");
             }
             if (n_active == 0) break;
-            k_convert<float2, double2><<<flat_grid(nt), 256, 0, s>>>((float2 *)S->rs.ptr, (const double2 *)S->r64.ptr, nt);
+            k_convert<<<dim3(flat_grid(n), R), 256, 0, s>>>((float2 *)S->rs.ptr, (const double2 *)S->r64.ptr, n, sc);
             for (int r = 0; r < R; ++r)
                 if (active[r] && (restart[r] || restart_all))
                     WEO_CUDA(cudaMemcpyAsync(static_cast<char *>(S->p.ptr) + r * v32,
