@@ -383,7 +383,10 @@ __global__ void __launch_bounds__(kRedThreads) k_residual_ff(double2 *r, const d
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (j > 0 && k0 + j * st >= n) break;
-            const double2 rv = make_double2(bv[j].x - ff_join(hi[j].x, lo[j].x), bv[j].y - ff_join(hi[j].y, lo[j].y));
+            // the two parts one after the other: b - hi is exact where they nearly cancel,
+            // so that no bit of lo is lost to the rounding of hi + lo
+            const double2 rv = make_double2((bv[j].x - double(hi[j].x)) - double(lo[j].x),
+                                            (bv[j].y - double(hi[j].y)) - double(lo[j].y));
             r[k0 + j * st] = rv;
             v += rv.x * rv.x + rv.y * rv.y;
         }
