@@ -169,10 +169,11 @@ __device__ __forceinline__ void hop_dir(cx<T> (&acc)[R][12], const HopParams &p,
 // The forward and backward hop of direction MU together (FP64, whose pipe
 // bounds these kernels: every operation saved is time saved). With P and Q the
 // two products W h, the upper rows receive P + Q and the lower ones -+S A^dag
-// (P - Q), because the backward projector has the opposite sign. The product Q
-// accumulates onto P, so P + Q costs no addition, and P - Q = 2 P - (P + Q) is
-// one fused operation: 48 FP64 operations fewer per site than two separate
-// reconstructions (and 24 more because nothing is added to zero).
+// (P - Q), because the backward projector has the opposite sign: one addition and
+// one subtraction where two separate reconstructions take two of each, and
+// nothing is added to zero (24 operations of 864 per site less). Accumulating Q
+// onto P and forming P - Q = 2 P - (P + Q) would save 48 more, but puts the
+// rounding of the sum into the lower rows: their error was 7-9 % larger.
 template <class SIn, class Lk, int MU, int S0, typename I>
 __device__ __forceinline__ void hop_pair(const HopParams &p, const char *in, I n_fwd, I n_bwd, I i,
                                          cx<double> sum[2][3], cx<double> dif[2][3])
@@ -197,12 +198,11 @@ __device__ __forceinline__ void hop_pair(const HopParams &p, const char *in, I n
     for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            cx<double> z = dif[s][a];
+            cx<double> z = {0.0, 0.0};
 #pragma unroll
             for (int b = 0; b < 3; ++b) z = cfmaconj(U[b][a], h[s][b], z);
-            sum[s][a] = z;
-            dif[s][a].r = fma(2.0, dif[s][a].r, -z.r);
-            dif[s][a].i = fma(2.0, dif[s][a].i, -z.i);
+            sum[s][a] = cadd(dif[s][a], z);
+            dif[s][a] = csub(dif[s][a], z);
         }
 }
 

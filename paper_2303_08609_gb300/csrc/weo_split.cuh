@@ -337,10 +337,10 @@ __device__ __forceinline__ void pair_rows(const HopParams &p, const char *in, co
         cx<double> P = {0.0, 0.0};
 #pragma unroll
         for (int c = 0; c < 3; ++c) P = cfma(Uf[k][c], h[c], P);
-        cx<double> z = P;
+        cx<double> Q = {0.0, 0.0};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) z = cfmaconj(Ub[c][k], g[c], z);
-        const cx<double> d = {fma(2.0, P.r, -z.r), fma(2.0, P.i, -z.i)};
+        for (int c = 0; c < 3; ++c) Q = cfmaconj(Ub[c][k], g[c], Q);
+        const cx<double> z = cadd(P, Q), d = csub(P, Q);
         part[16 * (3 * row + k)] = make_double2(z.r, z.i);
         cx<double> l = kRot ? cmuli(d) : d;
         if (neg) l = cneg(l);
