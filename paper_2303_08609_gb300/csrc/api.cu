@@ -143,9 +143,10 @@ static int upload_gauge(wilson_eo_s *h, const void *gauge, int gauge_is_f64, cud
 {
     const size_t bytes = (size_t)(2 * h->vh) * 4 * 9 * (gauge_is_f64 ? 16 : 8);
     WEO_TRY(h->canon_gauge.ensure(bytes));
-    // a field in this GPU's memory is copied by the packing kernel that reads it
-    // (one in another GPU's memory is not readable there without peer access)
-    const bool here = is_memory_of(gauge, h->device);
+    // a field in this GPU's memory is copied by the packing kernel that reads it (one
+    // in another GPU's memory is not readable there without peer access, one that
+    // does not start on a multiple of its reals' size not at all)
+    const bool here = reinterpret_cast<uintptr_t>(gauge) % (gauge_is_f64 ? 8 : 4) == 0 && is_memory_of(gauge, h->device);
     if (!here) {
         const cudaMemcpyKind kind =
             is_device_pointer(gauge) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
