@@ -268,8 +268,16 @@ __global__ void __launch_bounds__(128, 4) hop_kernel_ff(const HopParams p)
 template <bool Dag, bool Axpy, bool OutF64>
 static int launch_ff(const HopParams &p, cudaStream_t s)
 {
-    dim3 grid((unsigned)((p.vh + 31) / 32), (unsigned)p.nrhs);
-    return launch_dependent(hop_kernel_ff<Dag, Axpy, OutF64>, grid, 128, s, p);
+    const unsigned nsb = (unsigned)((p.vh + 31) / 32);
+    HopParams q = p;
+    for (long long r = 0; r < p.nrhs; r += kGridRows) {
+        q.nrhs = (int)(p.nrhs - r < kGridRows ? p.nrhs - r : kGridRows);
+        q.in = static_cast<const char *>(p.in) + r * p.in_stride;
+        q.out = static_cast<char *>(p.out) + r * p.out_stride;
+        if (Axpy) q.x = static_cast<const char *>(p.x) + r * p.x_stride;
+        WEO_TRY(launch_dependent(hop_kernel_ff<Dag, Axpy, OutF64>, dim3(nsb, (unsigned)q.nrhs), 128, s, q));
+    }
+    return WEO_OK;
 }
 
 int launch_hop_ff(bool dag, bool axpy, const HopParams &p, const LaunchCfg &, cudaStream_t s)

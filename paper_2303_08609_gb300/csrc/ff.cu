@@ -29,9 +29,13 @@ __global__ void __launch_bounds__(256) k_f64_to_ff(float2 *__restrict__ dst, con
 int ff_from_f64(void *dst, const void *src, long long vh, int nrhs, cudaStream_t s)
 {
     const long long per = 12 * vh;
-    const dim3 grid((unsigned)((per + 256 * kSplitPer - 1) / (256 * kSplitPer)), (unsigned)nrhs);
-    k_f64_to_ff<<<grid, 256, 0, s>>>(static_cast<float2 *>(dst), static_cast<const double2 *>(src), per);
-    WEO_CUDA(cudaGetLastError());
+    const unsigned blocks = (unsigned)((per + 256 * kSplitPer - 1) / (256 * kSplitPer));
+    for (long long r = 0; r < nrhs; r += kGridRows) {
+        const dim3 grid(blocks, (unsigned)(nrhs - r < kGridRows ? nrhs - r : kGridRows));
+        k_f64_to_ff<<<grid, 256, 0, s>>>(static_cast<float2 *>(dst) + r * 2 * per,
+                                         static_cast<const double2 *>(src) + r * per, per);
+        WEO_CUDA(cudaGetLastError());
+    }
     return WEO_OK;
 }
 

@@ -46,6 +46,11 @@ int launch_dependent(void (*kern)(K...), dim3 grid, unsigned block, cudaStream_t
     return WEO_OK;
 }
 
+// rows of a grid: more right-hand sides than these, one per row, take several launches
+// (a kernel that finds its right-hand side in a flat grid instead measured 302 to 308
+// against 297 us in the float-float hops at 24^3 x 48)
+constexpr int kGridRows = 65535;
+
 // ----------------------------------------------------------------- formats --
 // Internal operator precision next to weo_prec: float-float arithmetic with
 // 18-real links (FP64-class accuracy from FP32 operations); spinors SpFF.
