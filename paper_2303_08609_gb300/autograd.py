@@ -35,20 +35,25 @@ class MeoFunction(torch.autograd.Function):
     """chi = M_eo phi for the gauge field ``U`` (canonical ``(4, V, 3, 3)``).
 
     ``op`` is a :class:`WilsonEO` handle (FP64 or FP32) on the lattice of
-    ``U``; see :func:`_sync_gauge` for when its packed links are refreshed.
+    ``U``; see :func:`_sync_gauge` for when its packed links are refreshed. A 16-bit
+    handle computes the forward pass and the gradient of ``phi`` alone.
+    ``recorded``: whether a backward pass may follow (``needs_input_grad`` stays set
+    under ``torch.no_grad()``).
     """
 
     @staticmethod
-    def forward(ctx, phi, U, op, refresh=None):
+    def forward(ctx, phi, U, op, refresh=None, recorded=True):
         _sync_gauge(op, U, refresh)
         phi = phi.contiguous()
         ctx.op = op
         ctx.refresh = refresh
-        if not ctx.needs_input_grad[1] or phi.dim() != 3 or not phi.is_cuda:
+        # the link gradient needs the odd intermediate: where one may be asked for
+        # (16-bit handles have none), keep it, one spinor, rather than spend a third
+        # hop on it in the backward pass
+        if not (recorded and ctx.needs_input_grad[1] and op.prec in ("f64", "f32") and phi.dim() == 3
+                and phi.is_cuda):
             ctx.save_for_backward(phi, U)
             return op.apply(phi)
-        # the link gradient needs the odd intermediate: keep it, one spinor, rather
-        # than spend a third hop on it in the backward pass
         op._nrhs(phi)
         out, t = torch.empty_like(phi), torch.empty_like(phi)
         wilson_eo_grad_forward(op.handle, out, t, phi)
@@ -66,19 +71,19 @@ class MeoFunction(torch.autograd.Function):
             grad_phi = torch.empty_like(phi) if ctx.needs_input_grad[0] else None
             grad_U = torch.empty((4, 2 * op.vh, 3, 3), dtype=op.spinor_dtype(), device=phi.device)
             wilson_eo_grad_backward(op.handle, grad_phi, grad_U, g, phi, mid[0])
-            return grad_phi, grad_U, None, None
+            return grad_phi, grad_U, None, None, None
         grad_phi = op.apply(g, dag=True) if ctx.needs_input_grad[0] else None
         grad_U = None
         if ctx.needs_input_grad[1]:
             if phi.dim() != 3:
                 raise NotImplementedError("link gradient is provided for one right-hand side")
             grad_U = op.link_grad(g, phi)
-        return grad_phi, grad_U, None, None
+        return grad_phi, grad_U, None, None, None
 
 
 def meo(phi: torch.Tensor, U: torch.Tensor, op: WilsonEO, refresh=None) -> torch.Tensor:
     """Differentiable M_eo phi (see :class:`MeoFunction`)."""
-    return MeoFunction.apply(phi, U, op, refresh)
+    return MeoFunction.apply(phi, U, op, refresh, torch.is_grad_enabled())
 
 
 def pseudofermion_action(phi: torch.Tensor, U: torch.Tensor, op: WilsonEO,
