@@ -145,8 +145,8 @@ int wilson_eo_link_grad(wilson_eo_t h, void *grad, const void *g_e, const void *
  *                            hop the link gradient computes anyway
  * Two hops each instead of two and four. Results equal wilson_eo_apply,
  * wilson_eo_link_grad and wilson_eo_apply_dag. FP64 / FP32 handles, one right-hand
- * side, device arrays (WEO_ERR_ARG for host arrays or an output that aliases an
- * input); asynchronous on `stream`. */
+ * side, device arrays (WEO_ERR_ARG for host arrays or an output that overlaps an
+ * input or the other output); asynchronous on `stream`. */
 int wilson_eo_grad_forward(wilson_eo_t h, void *out_e, void *t_o, const void *in_e, void *stream);
 int wilson_eo_grad_backward(wilson_eo_t h, void *grad_phi, void *grad_gauge, const void *g_e,
                             const void *phi_e, const void *t_o, void *stream);

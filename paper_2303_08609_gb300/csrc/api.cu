@@ -119,6 +119,13 @@ static int finish_out(void *host_ptr, const void *dev, size_t bytes, bool host, 
     return WEO_OK;
 }
 
+// do the n_a bytes from a on and the n_b bytes from b on share one?
+static bool overlap(const void *a, size_t n_a, const void *b, size_t n_b)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + n_b && y < x + n_a;
+}
+
 // bytes of one external (canonical) spinor of the handle
 static size_t ext_spinor_bytes(const wilson_eo_s *h)
 {
@@ -715,7 +722,9 @@ int wilson_eo_grad_forward(wilson_eo_t h, void *out_e, void *t_o, const void *in
 {
     try {
         if (!h || !out_e || !t_o || !in_e) return set_error(WEO_ERR_ARG, "NULL handle or array");
-        if (out_e == in_e || t_o == in_e || t_o == out_e) return set_error(WEO_ERR_ARG, "arrays must not alias");
+        const size_t sb = ext_spinor_bytes(h);
+        if (overlap(out_e, sb, in_e, sb) || overlap(t_o, sb, in_e, sb) || overlap(t_o, sb, out_e, sb))
+            return set_error(WEO_ERR_ARG, "arrays must not overlap");
         if (h->prec != WEO_F64 && h->prec != WEO_F32)
             return set_error(WEO_ERR_UNSUPPORTED, "the gradient needs an FP64 or FP32 handle");
         if (!is_device_pointer(out_e) || !is_device_pointer(t_o) || !is_device_pointer(in_e))
@@ -723,7 +732,7 @@ int wilson_eo_grad_forward(wilson_eo_t h, void *out_e, void *t_o, const void *in
         DeviceGuard dg(h->device);
         Buffer mid;  // the caller's array in the place of the handle's intermediate
         mid.ptr = t_o;
-        mid.bytes = ext_spinor_bytes(h);
+        mid.bytes = sb;
         return meo_with(h, h->gauge, mid, out_e, in_e, 1, false, static_cast<cudaStream_t>(stream));
     } catch (...) {
         return set_error(WEO_ERR_OOM, "host exception in wilson_eo_grad_forward");
@@ -735,8 +744,11 @@ int wilson_eo_grad_backward(wilson_eo_t h, void *grad_phi, void *grad_gauge, con
 {
     try {
         if (!h || !grad_gauge || !g_e || !phi_e || !t_o) return set_error(WEO_ERR_ARG, "NULL handle or array");
-        if (grad_phi && (grad_phi == g_e || grad_phi == phi_e || grad_phi == t_o))
-            return set_error(WEO_ERR_ARG, "grad_phi must not alias an input");
+        const size_t sb = ext_spinor_bytes(h), gb = 6 * sb;  // 4 links of 9 for 12 values of a spinor, on both parities
+        for (const void *q : {g_e, phi_e, t_o, static_cast<const void *>(grad_phi)})
+            if (q && overlap(grad_gauge, gb, q, sb)) return set_error(WEO_ERR_ARG, "grad_gauge overlaps another array");
+        for (const void *q : {g_e, phi_e, t_o})
+            if (grad_phi && overlap(grad_phi, sb, q, sb)) return set_error(WEO_ERR_ARG, "grad_phi overlaps an input");
         if (h->prec != WEO_F64 && h->prec != WEO_F32)
             return set_error(WEO_ERR_UNSUPPORTED, "the gradient needs an FP64 or FP32 handle");
         const void *ptrs[4] = {grad_gauge, g_e, phi_e, t_o};
