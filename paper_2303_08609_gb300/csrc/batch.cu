@@ -195,9 +195,9 @@ static int launch_batch(void (*kern)(const BatchArgs), int threads, size_t smem,
 }
 
 template <class Lk>
-static int launch_batch_f32(const BatchArgs &a, bool dag, bool multi, cudaStream_t s)
+static int launch_batch_f32(const BatchArgs &a, bool dag, bool tiles, cudaStream_t s)
 {
-    if (multi)  // tiles with their links in shared memory for all right-hand sides
+    if (tiles)
         return launch_batch(dag ? batch_meo_tiles_kernel<Lk, true> : batch_meo_tiles_kernel<Lk, false>,
                             kLinkTile * kLinkGroups, (size_t)576 * kLinkTile, a.lt_begin[a.n], a, s);
     return launch_batch(dag ? batch_meo_kernel<Lk, true> : batch_meo_kernel<Lk, false>, kBatchThreads, 0,
@@ -234,6 +234,11 @@ static int apply_batch_impl(int n, const wilson_eo_t *hs, void *const *outs, con
     if (prec != WEO_F32 && prec != WEO_F64)
         return set_error(WEO_ERR_UNSUPPORTED, "batches are provided for FP64 and FP32 handles");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // FP32: tiles with their links in shared memory for all right-hand sides, whose
+    // offsets are 64 bits wide, also for lattices beyond the split blocks' offsets.
+    // (FP64 handles of that size, 206 GB of links with 12 reals beside a canonical field
+    // of 155 GB, do not fit the GPU.)
+    bool tiles = max_rhs >= 2;
     BatchArgs a;
     memset(&a, 0, sizeof(a));
     a.n = n;
@@ -258,7 +263,10 @@ static int apply_batch_impl(int n, const wilson_eo_t *hs, void *const *outs, con
         p.x = ins[k];
         p.a = -h->kappa * h->kappa;
         a.second[k] = p;
-        if (h->vh > (1ll << 28)) return set_error(WEO_ERR_UNSUPPORTED, "batched lattices hold at most 2^28 sites of a parity");
+        if (h->vh > kSplitMaxSites) {
+            if (prec == WEO_F64) return set_error(WEO_ERR_UNSUPPORTED, "FP64 batches hold at most 2^28 sites of a parity");
+            tiles = true;
+        }
         a.tile_begin[k + 1] = a.tile_begin[k] + (h->vh + 31) / 32 * nr;
         a.lt_begin[k + 1] = a.lt_begin[k] + (h->vh + kLinkTile - 1) / kLinkTile;
     }
@@ -268,8 +276,8 @@ static int apply_batch_impl(int n, const wilson_eo_t *hs, void *const *outs, con
     if (prec == WEO_F64)
         st = c ? launch_batch_f64<LkF64_12>(a, dag != 0, s) : launch_batch_f64<LkF64_18>(a, dag != 0, s);
     else
-        st = c ? launch_batch_f32<LkF32_12>(a, dag != 0, max_rhs >= 2, s)
-               : launch_batch_f32<LkF32_18>(a, dag != 0, max_rhs >= 2, s);
+        st = c ? launch_batch_f32<LkF32_12>(a, dag != 0, tiles, s)
+               : launch_batch_f32<LkF32_18>(a, dag != 0, tiles, s);
     prof_end(hs[0], tok, s);
     return st;
 }

@@ -40,9 +40,7 @@ int launch_tile_links(const HopParams &p, cudaStream_t s)
     return WEO_OK;
 }
 
-// Largest V/2 of the split kernels: their 32-bit offsets address 16-byte elements.
-constexpr int kSplitMaxSites = 1 << 28;
-// ... and with 12-real 16-bit links, times the right-hand sides: they issue the
+// With 12-real 16-bit links, times the right-hand sides: they issue the
 // most instructions per byte, and once the work fills the GPU many times over the
 // one-site kernel's fewer ones win. One site per thread : split, us per M_eo with
 // FP16: 62.2 : 57.5 at V/2 = 331776, 166 : 166 at 1048576, 788 : 817 at 5308416;

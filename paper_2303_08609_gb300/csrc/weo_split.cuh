@@ -35,6 +35,9 @@
 
 namespace weo {
 
+// Largest V/2 of these kernels: their 32-bit offsets address 16-byte elements.
+constexpr int kSplitMaxSites = 1 << 28;
+
 // chi = W h of one direction for one site, two spin rows x three colours
 template <int MU, bool FWD, int S0, class N>
 __device__ __forceinline__ void dir_chi(const cx<float> U[3][3], const cx<float> v[12], N scale, float2 *out)
