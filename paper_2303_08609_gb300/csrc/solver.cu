@@ -71,8 +71,7 @@ struct SolverState {
     cudaStream_t side = nullptr;               // reductions that overlap the operator
     cudaEvent_t fork = nullptr, join = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // [mixed]
-    int graph_chunk[2] = {0, 0};
-    int graph_nrhs[2] = {0, 0};
+    std::string graph_key[2];                       // what each was captured with
     double delta = 0.1;
     int chunk = 8;
     int use_graphs = 1;
@@ -570,6 +569,24 @@ static int cg_iteration(wilson_eo_s *h, SolverState *S, const PackedGauge &g, bo
                  : cg_step<double2>(h, S, g, S->odd64, S->x64.ptr, S->r64.ptr, S->p64.ptr, S->e64.ptr, S->Ap64.ptr, s);
 }
 
+// Everything that k captured iterations hold: numbers passed to the kernels, what
+// chooses the kernels, and the addresses of all arrays. A set_kappa, another launch
+// setting, or a buffer that grew for another solve make it another graph.
+static std::string graph_key(const wilson_eo_s *h, const SolverState *S, const PackedGauge &g, int k)
+{
+    std::string key;
+    auto add = [&](auto v) { key.append(reinterpret_cast<const char *>(&v), sizeof v); };
+    const LaunchCfg &c = h->cfg[g.prec];
+    add(h->kappa);
+    for (int v : {k, S->nrhs, h->algo, h->alternate, h->fused_lookahead, h->fused_threads, h->staged_rows, h->staged_depth,
+                  c.threads, c.rhs_block, c.lanes, c.staged, c.tile_links, c.tile_rhs_per_thread, c.blocked})
+        add(v);
+    for (const Buffer *b : {&g.buf, &S->scal, &S->xs, &S->rs, &S->p, &S->Ap, &S->t32, &S->oddlo, &S->x64, &S->r64,
+                            &S->p64, &S->Ap64, &S->e64, &S->odd64, &h->staged_links, &h->fs_links, &h->fused_ctrl})
+        add(b->ptr);
+    return key;
+}
+
 // Run `k` iterations, from a captured graph when enabled.
 static int cg_chunk(wilson_eo_s *h, SolverState *S, const PackedGauge &g, bool mixed, int k)
 {
@@ -579,7 +596,8 @@ static int cg_chunk(wilson_eo_s *h, SolverState *S, const PackedGauge &g, bool m
         return WEO_OK;
     }
     const int gi = mixed ? 1 : 0;
-    if (!S->graph[gi] || S->graph_chunk[gi] != k || S->graph_nrhs[gi] != S->nrhs) {
+    const std::string key = graph_key(h, S, g, k);
+    if (!S->graph[gi] || S->graph_key[gi] != key) {
         if (S->graph[gi]) {
             cudaGraphExecDestroy(S->graph[gi]);
             S->graph[gi] = nullptr;
@@ -608,8 +626,7 @@ static int cg_chunk(wilson_eo_s *h, SolverState *S, const PackedGauge &g, bool m
             S->graph[gi] = nullptr;
             return fail_cuda(e, "cudaGraphInstantiate", __FILE__, __LINE__);
         }
-        S->graph_chunk[gi] = k;
-        S->graph_nrhs[gi] = S->nrhs;
+        S->graph_key[gi] = key;
     }
     WEO_CUDA(cudaGraphLaunch(S->graph[gi], s));
     return WEO_OK;
