@@ -40,26 +40,6 @@ int launch_tile_links(const HopParams &p, cudaStream_t s)
     return WEO_OK;
 }
 
-// With 12-real 16-bit links, times the right-hand sides: they issue the
-// most instructions per byte, and once the work fills the GPU many times over the
-// one-site kernel's fewer ones win. One site per thread : split, us per M_eo with
-// FP16: 62.2 : 57.5 at V/2 = 331776, 166 : 166 at 1048576, 788 : 817 at 5308416;
-// at 331776 with 2 and 3 right-hand sides 105 : 107 and 149 : 155.
-constexpr long long kSplit16MaxSites = 3 << 18;
-// Several right-hand sides, unless the handle names a kernel: tiles whose links
-// sit in shared memory for four at a time pay from this many (site, right-hand
-// side) pairs on, and when their passes are well filled. Tiles : split, us per
-// M_eo with FP32 18-real links: 16^3 x 32 (V/2 = 65536) 4 RHS 51.8 : 49.8, 12 RHS
-// 119 : 136; 24^3 x 48 (331776) 3 RHS 194 : 185, 4 RHS 217 : 241, 5 RHS 299 : 295,
-// 12 RHS 520 : 670 (720 with one site per thread); 8^4 12 RHS 21.5 : 7.2. FP16
-// 12-real at 24^3 x 48: 4 RHS 197 : 195, 5 RHS 277 : 238, 12 RHS 478 : 546 (one
-// site per thread).
-constexpr long long kTileMinWork = 1 << 19;
-template <bool F16>
-inline bool tiles_pay(const HopParams &p)
-{
-    return p.nrhs >= (F16 ? 6 : 4) && p.nrhs != 5 && (long long)p.vh * p.nrhs >= kTileMinWork;
-}
 // FP64: below this many sites the 32-site CTAs of hop_kernel_pairs would leave
 // SMs idle (152 of them), and hop_kernel_rows' 16-site ones are faster: 11.9
 // against 17.5 us per M_eo at V/2 = 2048, but 34.4 against 31.5 at 7560 and 981
@@ -114,14 +94,14 @@ int launch_instance(const HopParams &p, const LaunchCfg &cfg, cudaStream_t s)
         if (nl == 8) return launch_lanes<SIn, SOut, SX, Lk, Dag, Axpy, 8>(p, cfg, s);
         if (nl == 4) return launch_lanes<SIn, SOut, SX, Lk, Dag, Axpy, 4>(p, cfg, s);
         if (nl == 2) return launch_lanes<SIn, SOut, SX, Lk, Dag, Axpy, 2>(p, cfg, s);
-        if (!cfg.blocked && tiles_pay<(Is16<SIn>::value || Is16<SOut>::value)>(p))
-            return launch_tile_links<SIn, SOut, SX, Lk, Dag, Axpy, 4>(p, s);
     }
-    // a site's directions on different warps
     if constexpr (R == 1) {
-        const bool fits = p.vh <= kSplitMaxSites &&
-                          (Lk::kBytesPerSite != 24 || (long long)p.vh * p.nrhs <= kSplit16MaxSites);
-        if (!cfg.blocked && fits) return launch_split<SIn, SOut, SX, Lk, Dag, Axpy>(p, s);
+        constexpr bool kF64 = sizeof(typename SOut::real) == 8, k16 = Is16<SIn>::value || Is16<SOut>::value;
+        constexpr bool k12 = Lk::kBytesPerSite == (kF64 ? 96 : k16 ? 24 : 48);
+        const Route route = cfg.blocked ? Route::OneSite : default_route(kF64, k16, k12, p.vh, p.nrhs);
+        if constexpr (!kF64)
+            if (route == Route::Tiles) return launch_tile_links<SIn, SOut, SX, Lk, Dag, Axpy, 4>(p, s);
+        if (route == Route::Split) return launch_split<SIn, SOut, SX, Lk, Dag, Axpy>(p, s);
     }
     // blocked site order: CTAs of 8 Lx/2 threads, one per 2x2x2 block of rows
     const bool blocked = cfg.blocked && 8 * p.lxh >= 64 && 8 * p.lxh <= 256;

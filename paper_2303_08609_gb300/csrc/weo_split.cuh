@@ -32,11 +32,9 @@
 #pragma once
 
 #include "weo_dslash.cuh"
+#include "weo_route.h"
 
 namespace weo {
-
-// Largest V/2 of these kernels: their 32-bit offsets address 16-byte elements.
-constexpr int kSplitMaxSites = 1 << 28;
 
 // chi = W h of one direction for one site, two spin rows x three colours
 template <int MU, bool FWD, int S0, class N>

@@ -1,0 +1,138 @@
+"""The kernel that a call takes by default (``csrc/weo_route.h``), compiled alone.
+
+``MEASURED`` has us per M_eo on one GB300 of every kernel the rules choose between: the
+chosen one is at most 3 % slower than the fastest, so that no rule sends a size to a
+kernel which its own measurement shows to be the slower one.
+"""
+
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2303_08609_gb300", "csrc")
+
+# bits, link reals, V/2, right-hand sides: one site per thread, split, tiles
+MEASURED = """
+16 12 65536 2 26.75 23.47 32.60
+16 12 65536 8 84.54 83.24 78.02
+16 12 65536 9 93.09 92.76 96.91
+16 12 65536 10 101.26 102.23 100.38
+16 12 65536 12 119.07 121.37 109.45
+16 12 65536 13 127.97 130.99 128.15
+16 12 331776 2 106.94 106.45 147.34
+16 12 331776 3 151.26 155.21 178.55
+16 12 331776 4 196.17 204.05 195.93
+16 12 331776 5 240.97 252.99 275.93
+16 12 331776 6 285.53 301.80 291.99
+16 12 331776 7 329.99 350.66 322.16
+16 12 331776 9 419.06 448.34 411.90
+16 12 331776 12 552.59 594.85 479.49
+16 12 32768 16 83.81 83.04 84.80
+16 12 131072 4 85.48 84.15 83.03
+16 12 131072 6 119.96 122.10 122.34
+16 12 262144 3 121.88 123.40 999
+16 12 331776 1 62.83 56.46 999
+16 12 589824 1 101.44 96.73 999
+16 12 589824 2 179.20 185.00 999
+16 12 1048576 1 168.36 165.59 999
+16 12 1048576 2 306.75 323.17 999
+16 12 5308416 1 788 817 9999
+16 18 65536 5 60.58 51.62 64.22
+16 18 65536 8 84.77 79.51 78.60
+16 18 65536 9 91.29 88.52 97.70
+16 18 65536 10 102.26 97.37 101.31
+16 18 65536 12 120.21 115.42 110.08
+16 18 65536 13 126.52 124.29 129.00
+16 18 331776 3 155.01 150.45 180.10
+16 18 331776 4 197.25 196.54 197.51
+16 18 331776 5 239.86 242.94 277.96
+16 18 331776 6 282.79 289.23 294.00
+16 18 331776 7 325.61 335.56 324.19
+16 18 331776 9 411.34 428.30 414.44
+16 18 331776 10 454.24 474.72 434.17
+16 18 331776 13 581.70 613.78 550.33
+16 18 32768 16 83.37 79.13 85.40
+16 18 131072 4 87.80 80.72 83.98
+16 18 131072 6 123.35 116.78 123.36
+16 18 5308416 1 867 851 9999
+32 18 65536 4 59.24 50.35 51.65
+32 18 65536 8 108.05 94.58 84.58
+32 18 65536 9 115.49 104.52 105.11
+32 18 65536 13 161.24 146.78 137.32
+32 18 331776 3 207.14 188.25 192.44
+32 18 331776 4 261.78 243.11 215.43
+32 18 331776 5 317.00 297.25 295.06
+32 18 331776 6 373.46 351.83 314.36
+32 18 331776 9 537.62 516.52 440.47
+32 18 32768 16 104.79 92.39 93.07
+32 18 131072 4 113.47 98.47 92.01
+32 18 131072 6 160.84 141.21 130.85
+32 12 65536 8 99.90 86.62 82.58
+32 12 65536 9 112.56 96.58 103.39
+32 12 65536 10 118.24 106.51 106.37
+32 12 65536 13 151.20 136.36 135.87
+32 12 331776 4 245.61 220.77 208.29
+32 12 331776 5 302.01 271.99 289.95
+32 12 331776 6 355.33 323.43 308.65
+32 12 331776 9 523.17 477.03 436.03
+32 12 32768 16 97.32 85.83 91.81
+32 12 131072 6 148.10 128.11 127.69
+"""
+
+
+@pytest.fixture(scope="module")
+def route(tmp_path_factory):
+    """(bits, reals, V/2, nrhs) -> 0 one site, 1 split, 2 tiles"""
+    gxx = shutil.which("g++") or pytest.skip("no g++")
+    d = tmp_path_factory.mktemp("route")
+    src = d / "route.cc"
+    src.write_text('#include <cstdio>\n#include "weo_route.h"\nint main() { int b, l, n; long long v;\n'
+                   'while (scanf("%d %d %lld %d", &b, &l, &v, &n) == 4)\n'
+                   'printf("%d\\n", (int)weo::default_route(b == 64, b == 16, l == 12, v, n)); }\n')
+    subprocess.run([gxx, "-std=c++17", "-I", CSRC, str(src), "-o", str(d / "route")], check=True)
+
+    def ask(rows):
+        text = "\n".join(" ".join(map(str, r)) for r in rows)
+        return list(map(int, subprocess.run([str(d / "route")], input=text, capture_output=True, text=True,
+                                            check=True).stdout.split()))
+
+    return ask
+
+
+def test_the_chosen_kernel_is_the_measured_one(route):
+    rows = [line.split() for line in MEASURED.split("\n") if line]
+    for r, got in zip(rows, route([r[:4] for r in rows])):
+        us = list(map(float, r[4:]))
+        assert us[got] <= 1.03 * min(us), r
+
+
+def test_offsets_of_the_split_kernels(route):
+    """Beyond 2^28 sites, where 32-bit offsets end, nothing takes them."""
+    rows = [(b, l, v, n) for b in (64, 32, 16) for l in (18, 12) for v in (2 ** 28 + 1, 2 ** 31 - 1) for n in (1, 2, 3, 5, 8)]
+    assert 1 not in route(rows)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec,fmt,counts", [("f16", 12, (2, 3, 4, 5, 6, 7)), ("bf16", 18, (3, 5, 6, 7)),
+                                             ("f32", 18, (3, 4, 5)), ("f32", 12, (4, 5))])
+def test_right_hand_sides_on_both_sides_of_the_rules(prec, fmt, counts):
+    """V/2 = 331776, where these counts cross the rules: each right-hand side is bitwise
+    the single one (split for FP32 and 18-real links; 12-real 16-bit ones too)."""
+    import torch
+
+    import paper_2303_08609_gb300 as weo
+
+    dims, n = (24, 24, 24, 48), max(counts)
+    g = torch.Generator(device="cuda").manual_seed(1101)
+    V = int(np.prod(dims))
+    # any links do: the kernels are compared with one another
+    U = 0.4 * torch.randn(4, V, 3, 3, dtype=torch.complex64, device="cuda", generator=g)
+    x = torch.randn(n, 4, 3, V // 2, dtype=torch.complex64, device="cuda", generator=g)
+    with weo.WilsonEO(dims, 0.13, U, prec=prec, linkfmt=fmt) as op:
+        for dag in (False, True):
+            one = torch.stack([op.apply(x[r].contiguous(), dag=dag) for r in range(n)])
+            for k in counts:
+                assert torch.equal(op.apply(x[:k].contiguous(), dag=dag), one[:k])
