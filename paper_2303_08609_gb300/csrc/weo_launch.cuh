@@ -40,14 +40,6 @@ int launch_tile_links(const HopParams &p, cudaStream_t s)
     return WEO_OK;
 }
 
-// FP64: below this many sites the 32-site CTAs of hop_kernel_pairs would leave
-// SMs idle (152 of them), and hop_kernel_rows' 16-site ones are faster: 11.9
-// against 17.5 us per M_eo at V/2 = 2048, but 34.4 against 31.5 at 7560 and 981
-// against 927 at 331776. With 12-real links both half-warps would rebuild the
-// third row, on the pipe that bounds the kernel (16.3 against 21.7 us at 2048
-// sites, 49.9 against 40.2 at 7560).
-constexpr int kRowsMaxSites = 32 * 152;
-
 // Directions on the warps of a CTA (weo_split.cuh). Resident CTAs per SM that
 // the registers are held to, us per M_eo at 32^3 x 64 with 8 / 9 / 10 of them (64,
 // 56, 48 registers): FP32 18-real 241 / 242 / 262 (spills), FP32 12-real
@@ -57,7 +49,7 @@ int launch_split(const HopParams &p, cudaStream_t s)
 {
     const unsigned nsb = (unsigned)((p.vh + 31) / 32);
     if constexpr (std::is_same<typename SOut::real, double>::value) {
-        if (p.vh < kRowsMaxSites)
+        if (rows_pay(Lk::kBytesPerSite == 96, p.vh, p.nrhs))
             return launch_dependent(hop_kernel_rows<Lk, Dag, Axpy>, (unsigned)((p.vh + 15) / 16) * p.nrhs, 128, s, p);
         return launch_dependent(hop_kernel_pairs<Lk, Dag, Axpy>, nsb * p.nrhs, 128, s, p);
     } else {

@@ -55,6 +55,23 @@ inline bool split_pays(bool bits16, bool link12, long long vh, int nrhs)
     return vh * nrhs <= (link12 ? 5 << 17 : 5 << 18);
 }
 
+// FP64: hop_kernel_rows (16-site CTAs) in the place of hop_kernel_pairs (32 sites). Both
+// are bound by the FP64 pipe of each of the 152 SMs, so what counts is how many CTAs the
+// fullest SM gets: an odd number of 16-site ones is less work for it than the next 32-site
+// one, until the rows' 3 to 6 % of overhead outweigh the half CTA saved; with 12-real
+// links both half-warps rebuild the third row, which costs more. Rows : pairs, us per
+// M_eo, by 16-site CTAs per SM:
+//   18-real: 1 8^4 15.2 : 18.3; 2 8^3 x 16 22.6 : 18.7, 8^4 2 RHS 22.2 : 18.6; 3 8^4 3 RHS
+//     28.0 : 32.8; 4 10x6x14x18 35.2 : 33.2; 6 8^3 x 12 4 RHS 49.5 : 47.5; 7 8^3 x 16 4 RHS
+//     57.5 : 62.1; 11 8^4 12 RHS 87.6 : 90.0; 13 10x6x14x18 4 RHS 103 : 105; 38 293 : 279
+//   12-real: 1 8^4 19.9 : 21.5; 2 8^3 x 12 24.8 : 21.7; 3 8^4 3 RHS 37.4 : 39.6; 4 46.6 : 39.7;
+//     7 8^3 x 16 4 RHS 78.8 : 75.2; 11 8^4 12 RHS 121 : 109
+inline bool rows_pay(bool link12, long long vh, int nrhs)
+{
+    const long long per_sm = ((vh + 15) / 16 * nrhs + 151) / 152;
+    return per_sm % 2 == 1 && per_sm <= (link12 ? 3 : 7);
+}
+
 inline Route default_route(bool f64, bool bits16, bool link12, long long vh, int nrhs)
 {
     if (f64) return vh <= kSplitMaxSites ? Route::Split : Route::OneSite;

@@ -11,7 +11,7 @@ from lattice_ref import GAMMA, parity_sites, shift_index
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (10, 8, 10, 14)])  # both sides of V/2 = 4864
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (8, 8, 8, 16)])  # 16-site and 32-site CTAs
 @pytest.mark.parametrize("mu", range(4))
 @pytest.mark.parametrize("dag", [False, True])
 def test_difference_is_not_taken_from_the_sum(dims, mu, dag):

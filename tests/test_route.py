@@ -82,16 +82,61 @@ MEASURED = """
 32 12 131072 6 148.10 128.11 127.69
 """
 
+# FP64: link reals, V/2, right-hand sides: rows (16-site CTAs), pairs (32 sites)
+MEASURED_F64 = """
+18 256 1 11.36 17.46
+18 256 4 11.57 18.15
+18 256 12 18.93 18.43
+18 2048 1 15.23 18.32
+18 2048 2 22.24 18.60
+18 2048 3 27.97 32.79
+18 2048 4 34.95 32.88
+18 2048 12 87.63 89.99
+18 3072 1 18.96 18.44
+18 3072 2 28.45 32.72
+18 3072 3 34.98 32.98
+18 3072 4 49.48 47.50
+18 3072 12 125.76 119.44
+18 4096 1 22.60 18.65
+18 4096 2 34.97 32.90
+18 4096 3 49.47 47.49
+18 4096 4 57.50 62.05
+18 4608 1 22.80 18.75
+18 4608 4 65.28 62.28
+18 7560 1 35.20 33.19
+18 7560 2 57.57 62.26
+18 7560 3 80.29 76.11
+18 7560 4 103.36 105.05
+18 7560 12 293.47 278.71
+12 256 1 14.77 21.13
+12 256 12 24.72 21.67
+12 2048 1 19.87 21.52
+12 2048 2 30.00 21.89
+12 2048 3 37.36 39.63
+12 2048 4 46.56 39.68
+12 2048 12 121.42 109.13
+12 3072 1 24.76 21.68
+12 3072 2 37.85 39.65
+12 3072 3 46.59 39.78
+12 4096 1 30.03 21.88
+12 4096 4 78.79 75.18
+12 4608 4 89.42 75.36
+12 7560 1 46.55 39.90
+12 7560 2 78.74 75.52
+12 7560 12 411.68 338.47
+"""
+
 
 @pytest.fixture(scope="module")
 def route(tmp_path_factory):
-    """(bits, reals, V/2, nrhs) -> 0 one site, 1 split, 2 tiles"""
+    """(bits, reals, V/2, nrhs) -> 0 one site, 1 split (bits 64: 4 its rows kernel), 2 tiles"""
     gxx = shutil.which("g++") or pytest.skip("no g++")
     d = tmp_path_factory.mktemp("route")
     src = d / "route.cc"
     src.write_text('#include <cstdio>\n#include "weo_route.h"\nint main() { int b, l, n; long long v;\n'
                    'while (scanf("%d %d %lld %d", &b, &l, &v, &n) == 4)\n'
-                   'printf("%d\\n", (int)weo::default_route(b == 64, b == 16, l == 12, v, n)); }\n')
+                   'printf("%d\\n", b == 64 && weo::rows_pay(l == 12, v, n) ? 4 :\n'
+                   '       (int)weo::default_route(b == 64, b == 16, l == 12, v, n)); }\n')
     subprocess.run([gxx, "-std=c++17", "-I", CSRC, str(src), "-o", str(d / "route")], check=True)
 
     def ask(rows):
@@ -109,10 +154,37 @@ def test_the_chosen_kernel_is_the_measured_one(route):
         assert us[got] <= 1.03 * min(us), r
 
 
+def test_rows_and_pairs_are_the_measured_ones(route):
+    rows = [line.split() for line in MEASURED_F64.split("\n") if line]
+    for r, got in zip(rows, route([["64"] + r[:3] for r in rows])):
+        us = {4: float(r[3]), 1: float(r[4])}
+        assert us[got] <= 1.03 * min(us.values()), r
+
+
 def test_offsets_of_the_split_kernels(route):
     """Beyond 2^28 sites, where 32-bit offsets end, nothing takes them."""
     rows = [(b, l, v, n) for b in (64, 32, 16) for l in (18, 12) for v in (2 ** 28 + 1, 2 ** 31 - 1) for n in (1, 2, 3, 5, 8)]
     assert 1 not in route(rows)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fmt", [18, 12])
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (8, 8, 8, 16), (6, 10, 8, 14)])
+def test_fp64_rows_and_pairs_agree(dims, fmt):
+    """Counts that alternate between the two kernels, ragged against both CTA sizes."""
+    import torch
+
+    import paper_2303_08609_gb300 as weo
+
+    g = torch.Generator(device="cuda").manual_seed(1102)
+    V, n = int(np.prod(dims)), 7
+    U = 0.4 * torch.randn(4, V, 3, 3, dtype=torch.complex128, device="cuda", generator=g)
+    x = torch.randn(n, 4, 3, V // 2, dtype=torch.complex128, device="cuda", generator=g)
+    with weo.WilsonEO(dims, 0.13, U, prec="f64", linkfmt=fmt) as op:
+        for dag in (False, True):
+            one = torch.stack([op.apply(x[r].contiguous(), dag=dag) for r in range(n)])
+            for k in range(2, n + 1):
+                assert torch.equal(op.apply(x[:k].contiguous(), dag=dag), one[:k])
 
 
 @pytest.mark.gpu
