@@ -87,16 +87,16 @@ int launch_instance(const HopParams &p, const LaunchCfg &cfg, cudaStream_t s)
         if (nl == 4) return launch_lanes<SIn, SOut, SX, Lk, Dag, Axpy, 4>(p, cfg, s);
         if (nl == 2) return launch_lanes<SIn, SOut, SX, Lk, Dag, Axpy, 2>(p, cfg, s);
     }
+    // blocked site order: CTAs of 8 Lx/2 threads, one per 2x2x2 block of rows
+    const bool blocked = site_blocks_apply(cfg.blocked, p.lxh);
     if constexpr (R == 1) {
         constexpr bool kF64 = sizeof(typename SOut::real) == 8, k16 = Is16<SIn>::value || Is16<SOut>::value;
         constexpr bool k12 = Lk::kBytesPerSite == (kF64 ? 96 : k16 ? 24 : 48);
-        const Route route = cfg.blocked ? Route::OneSite : default_route(kF64, k16, k12, p.vh, p.nrhs);
+        const Route route = blocked ? Route::OneSite : default_route(kF64, k16, k12, p.vh, p.nrhs);
         if constexpr (!kF64)
             if (route == Route::Tiles) return launch_tile_links<SIn, SOut, SX, Lk, Dag, Axpy, 4>(p, s);
         if (route == Route::Split) return launch_split<SIn, SOut, SX, Lk, Dag, Axpy>(p, s);
     }
-    // blocked site order: CTAs of 8 Lx/2 threads, one per 2x2x2 block of rows
-    const bool blocked = cfg.blocked && 8 * p.lxh >= 64 && 8 * p.lxh <= 256;
     const int threads = blocked ? 8 * p.lxh : cfg.threads;
     const long long site_blocks = blocked ? (long long)(p.ly / 2) * (p.lz / 2) * (p.lt / 2)
                                           : (p.vh + threads - 1) / threads;

@@ -72,6 +72,10 @@ inline bool rows_pay(bool link12, long long vh, int nrhs)
     return per_sm % 2 == 1 && per_sm <= (link12 ? 3 : 7);
 }
 
+// The handle's 2x2x2 blocks of rows have CTAs of 8 Lx/2 threads, 64 to 256 of them; on
+// another lattice the setting changes nothing.
+inline bool site_blocks_apply(bool asked, int lxh) { return asked && 8 * lxh >= 64 && 8 * lxh <= 256; }
+
 inline Route default_route(bool f64, bool bits16, bool link12, long long vh, int nrhs)
 {
     if (f64) return vh <= kSplitMaxSites ? Route::Split : Route::OneSite;

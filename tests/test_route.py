@@ -161,6 +161,18 @@ def test_rows_and_pairs_are_the_measured_ones(route):
         assert us[got] <= 1.03 * min(us.values()), r
 
 
+def test_site_blocks_leave_other_lattices_alone(tmp_path):
+    """The setting holds from Lx = 16 to 64; elsewhere the default kernel stays."""
+    gxx = shutil.which("g++") or pytest.skip("no g++")
+    (tmp_path / "b.cc").write_text('#include "weo_route.h"\nint main(int n, char **v) { for (int l = 1; l < 100; ++l)\n'
+                                   'if (weo::site_blocks_apply(true, l) != (2 * l >= 16 && 2 * l <= 64) ||\n'
+                                   'weo::site_blocks_apply(false, l)) return 1; return 0; }\n')
+    subprocess.run([gxx, "-std=c++17", "-I", CSRC, str(tmp_path / "b.cc"), "-o", str(tmp_path / "b")], check=True)
+    assert subprocess.run([str(tmp_path / "b")]).returncode == 0
+    with open(os.path.join(CSRC, "weo_launch.cuh")) as f:
+        assert f.read().count("cfg.blocked") == 1  # only through the rule
+
+
 def test_offsets_of_the_split_kernels(route):
     """Beyond 2^28 sites, where 32-bit offsets end, nothing takes them."""
     rows = [(b, l, v, n) for b in (64, 32, 16) for l in (18, 12) for v in (2 ** 28 + 1, 2 ** 31 - 1) for n in (1, 2, 3, 5, 8)]
