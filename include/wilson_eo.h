@@ -275,9 +275,9 @@ int wilson_eo_apply_batch_rhs(int n, const wilson_eo_t *hs, void *const *outs,
 
 /* Autotune M_eo on this handle with nrhs right-hand sides: every candidate is
  * timed with CUDA events on `stream` and the fastest is kept -- the two-launch
- * algorithm with its default kernel, with threads 64/128/192/256 per CTA and 2 or
- * 4 right-hand sides per thread or 2 on neighbouring lanes (FP32 / 16-bit handles,
- * nrhs >= 2), and
+ * algorithm with its default kernel (with threads 64/128/192/256 per CTA where that
+ * computes a whole site in one thread), with those threads and 2 or 4 right-hand
+ * sides per thread or 2 on neighbouring lanes (FP32 / 16-bit handles, nrhs >= 2), and
  * for FP32 / 16-bit handles the fused algorithm with a lookahead of 4 or 8
  * t-slices and 128 / 256 threads, and for FP32 18-real handles with nrhs = 1
  * the TMA-staged hop (wilson_eo_get_launch, wilson_eo_get_algorithm,

@@ -1,10 +1,10 @@
 // Autotuner for M_eo: times each candidate on the handle's own lattice and
 // keeps the fastest. Candidates: the two-launch algorithm with its default kernel
-// and (FP32 / 16-bit handles with several right-hand sides) 64..256 threads per
-// CTA with 2 or 4 right-hand sides per thread, or two on neighbouring lanes,
-// or tiles whose links sit in shared memory for 2, 4 or 8 right-hand sides at
-// a time, or CTAs over 2x2x2 blocks of rows;
-// and, for FP32 / 16-bit handles, the fused single-launch algorithm with a
+// (with 64..256 threads per CTA where that is one site per thread) and (FP32 /
+// 16-bit handles with several right-hand sides) 64..256 threads per CTA with 2 or
+// 4 right-hand sides per thread, or two on neighbouring lanes, or tiles whose
+// links sit in shared memory for 2, 4 or 8 right-hand sides at a time, or CTAs
+// over 2x2x2 blocks of rows; and, for FP32 / 16-bit handles, the fused single-launch algorithm with a
 // lookahead of 4 or 8 t-slices and 128 or 256 threads per CTA; for FP32 18-real
 // handles the fused staged launch with a lookahead of 2 or 4. Results are
 // cached per process, keyed by (GPU name, extents, precision, link format,
@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "weo_internal.h"
+#include "weo_route.h"
 
 namespace weo {
 
@@ -161,8 +162,9 @@ int tune_handle(wilson_eo_s *h, int nrhs, cudaStream_t s, int *threads_out, int 
     std::vector<TuneEntry> cands;
     for (int threads : {64, 128, 192, 256}) {
         for (int r : rb) {
-            // one right-hand side per thread: the split hops, whose CTAs have one size
-            if (r == 1 && threads != 128) continue;
+            if (r == 1 && threads != 128 &&
+                !threads_matter(h->prec == WEO_F64, h->prec >= WEO_F16, h->fmt == WEO_LINK12, h->vh, nrhs))
+                continue;
             cands.push_back({0, threads, r, 1, 0, 0.0});
         }
         if (h->prec != WEO_F64 && nrhs >= 2) cands.push_back({0, threads, 1, 2, 0, 0.0});

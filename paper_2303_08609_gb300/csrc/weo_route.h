@@ -83,4 +83,11 @@ inline Route default_route(bool f64, bool bits16, bool link12, long long vh, int
     return split_pays(bits16, link12, vh, nrhs) ? Route::Split : Route::OneSite;
 }
 
+// whether the handle's threads per CTA reach the default kernel: the others have CTAs
+// of one size
+inline bool threads_matter(bool f64, bool bits16, bool link12, long long vh, int nrhs)
+{
+    return default_route(f64, bits16, link12, vh, nrhs) == Route::OneSite;
+}
+
 }  // namespace weo

@@ -173,6 +173,19 @@ def test_site_blocks_leave_other_lattices_alone(tmp_path):
         assert f.read().count("cfg.blocked") == 1  # only through the rule
 
 
+def test_tuner_times_thread_counts_where_they_matter(tmp_path):
+    """12-real 16-bit links at V/2 = 5308416 (48^3 x 96) run one site per thread."""
+    gxx = shutil.which("g++") or pytest.skip("no g++")
+    (tmp_path / "t.cc").write_text('#include "weo_route.h"\nint main() { using weo::threads_matter;\n'
+                                   'return !(threads_matter(false, true, true, 5308416, 1) && threads_matter(false, true, true, 331776, 3)\n'
+                                   '&& !threads_matter(false, true, true, 331776, 1) && !threads_matter(false, false, true, 5308416, 1)\n'
+                                   '&& !threads_matter(true, false, false, 331776, 1) && !threads_matter(false, true, false, 331776, 12)); }\n')
+    subprocess.run([gxx, "-std=c++17", "-I", CSRC, str(tmp_path / "t.cc"), "-o", str(tmp_path / "t")], check=True)
+    assert subprocess.run([str(tmp_path / "t")]).returncode == 0
+    with open(os.path.join(CSRC, "tune.cu")) as f:
+        assert "threads_matter(" in f.read()
+
+
 def test_offsets_of_the_split_kernels(route):
     """Beyond 2^28 sites, where 32-bit offsets end, nothing takes them."""
     rows = [(b, l, v, n) for b in (64, 32, 16) for l in (18, 12) for v in (2 ** 28 + 1, 2 ** 31 - 1) for n in (1, 2, 3, 5, 8)]
