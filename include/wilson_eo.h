@@ -284,7 +284,8 @@ int wilson_eo_apply_batch_rhs(int n, const wilson_eo_t *hs, void *const *outs,
  * wilson_eo_get_staging). threads_out / rhs_block_out describe the winner. Results
  * are cached per process by (GPU, extents, precision, link format, nrhs) and,
  * if the environment variable WILSON_EO_TUNE_CACHE names a file, appended to it
- * and read back by later processes. Allocates two temporary spinor fields.
+ * and read back by later processes (lines written by versions with other default
+ * kernels are passed over and timed again). Allocates two temporary spinor fields.
  * Any output pointer may be NULL. Blocks until done. */
 int wilson_eo_tune(wilson_eo_t h, int nrhs, int *threads_out, int *rhs_block_out, double *ms_out,
                    void *stream);
