@@ -132,7 +132,7 @@ def fields(seed=0):
 
 
 # sources that define the FP32 hopping kernels whose DRAM traffic ncu measured
-HOP_SOURCES = ("weo_fields.cuh", "weo_dslash.cuh", "weo_split.cuh", "weo_launch.cuh", "dslash_f32.cu")
+HOP_SOURCES = ("weo_fields.cuh", "weo_dslash.cuh", "weo_split.cuh", "weo_route.h", "weo_launch.cuh", "dslash_f32.cu")
 
 
 def sources_for(label):

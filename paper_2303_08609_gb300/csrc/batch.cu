@@ -39,8 +39,10 @@ __device__ __forceinline__ int find_lattice(const BatchArgs &a, long long tile)
 // One right-hand side per lattice: 32 sites at a time with their directions on the
 // CTA's four warps (weo_split.cuh). The second hop walks the tiles from the last to
 // the first, so it starts with the intermediates written last, still in L2.
-// 16^4 + 24^3 x 48 + 32^3 x 64, FP32 18-real: 345 us against 420 with one site per
-// thread (110 registers).
+// 16^4 + 24^3 x 48 + 32^3 x 64, FP32 18-real: 347 us against 420 with one site per
+// thread (110 registers); three separate calls take 330, since here every CTA waits
+// for the grid between the hops and the lattice's parameters, indexed at run time,
+// spill 44 bytes at 64 registers (18-real links).
 template <class Lk, bool Dag>
 __global__ void __launch_bounds__(kBatchThreads, 8) batch_meo_kernel(const __grid_constant__ BatchArgs a)
 {
@@ -86,7 +88,8 @@ __global__ void __launch_bounds__(kBatchThreads, 3) batch_meo_kernel_f64(const _
 // Several right-hand sides (FP32): the same cooperative walk over tiles of
 // 64 sites whose eight links per site are first copied into shared memory,
 // then used by all the lattice's right-hand sides, four at a time (one per
-// thread) -- the tile-shared-link hop of the single-lattice path.
+// thread) -- the tile-shared-link hop of the single-lattice path. The three lattices
+// above with four right-hand sides each: 1072 us, as separate calls 887.
 constexpr int kLinkTile = 64, kLinkGroups = 4;
 
 __device__ __forceinline__ int find_lattice_lt(const BatchArgs &a, long long tile)

@@ -282,9 +282,7 @@ __global__ void __launch_bounds__(4 * kGradSites, 3) link_grad_kernel_f64(const 
     T *dst = static_cast<T *>(p.out) + 18 * (w * V + lex0);
     if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
         // 16-byte vectors (n is even; the range starts 16-byte aligned whenever the output does)
-        using V4 = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-        constexpr int kPer = 16 / sizeof(T);
-        for (int k = lane; k < 18 * n / kPer; k += 32) reinterpret_cast<V4 *>(dst)[k] = reinterpret_cast<const V4 *>(sh)[k];
+        for (int k = lane; k < 9 * n; k += 32) reinterpret_cast<double2 *>(dst)[k] = reinterpret_cast<const double2 *>(sh)[k];
     } else {
         for (int k = lane; k < 18 * n; k += 32) dst[k] = sh[k];
     }

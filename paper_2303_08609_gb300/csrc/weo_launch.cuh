@@ -42,8 +42,8 @@ int launch_tile_links(const HopParams &p, cudaStream_t s)
 
 // Directions on the warps of a CTA (weo_split.cuh). Resident CTAs per SM that
 // the registers are held to, us per M_eo at 32^3 x 64 with 8 / 9 / 10 of them (64,
-// 56, 48 registers): FP32 18-real 241 / 242 / 262 (spills), FP32 12-real
-// 204 / 199 / 208, FP16 12-real 177 / 171 / 166, FP16 18-real 177 / 175 / 171.
+// 56, 48 registers): FP32 18-real 241 / 241 / 253 (spills), FP32 12-real
+// 202 / 196 / 201, FP16 12-real 176 / 170 / 165, FP16 18-real 175 / 174 / 170.
 template <class SIn, class SOut, class SX, class Lk, bool Dag, bool Axpy>
 int launch_split(const HopParams &p, cudaStream_t s)
 {

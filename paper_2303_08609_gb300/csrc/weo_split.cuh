@@ -16,19 +16,18 @@
 //
 // us per M_eo on one GB300, one site per thread -> split:
 //   lattice        FP32 18-real     FP32 12-real     FP16 18-real     FP64 18-real
-//   8^4            10.9 -> 4.0       8.6 -> 4.6       9.4 -> 4.9      63.7 -> 11.9
-//   16^3 x 32      25.4 -> 15.8     19.0 -> 14.6     20.0 -> 14.0      243 -> 195
-//   24^3 x 48       104 -> 78       77.0 -> 66.8     68.9 -> 57.4     1070 -> 927
-//   32^3 x 64       278 -> 241       227 -> 199       181 -> 171
-//   48^3 x 96      1358 -> 1206     1109 -> 991       867 -> 851
+//   8^4            10.9 -> 3.7       8.6 -> 4.1       9.4 -> 4.3      63.7 -> 12.6
+//   16^3 x 32      25.4 -> 15.5     19.0 -> 13.5     20.0 -> 13.2      243 -> 207
+//   24^3 x 48       104 -> 77       77.0 -> 65.2     68.9 -> 56.6     1070 -> 996
+//   32^3 x 64       278 -> 240       227 -> 196       181 -> 171
+//   48^3 x 96      1358 -> 1205     1109 -> 977       867 -> 848
 // CTAs of 64 or 128 sites measured slower (249 and 261 us at 32^3 x 64, FP32
 // 18-real), and so did both spin rows of a colour as one 16-byte value (257:
 // spills).
 // FP32 18-real links: bound by HBM (7.1 TB/s of the two passes' 816 B per site at
 // 32^3 x 64; the copy bandwidth is 6.8, part of the intermediate stays in L2).
 // 12-real and 16-bit links: instruction issue (68-72 % of cycles at 32^3 x 32 with
-// FP16) and the L1 / shared-memory path (57-76 %) together. FP64: the FP64 pipe
-// (97 % of its measured FMA rate at 24^3 x 48).
+// FP16) and the L1 / shared-memory path (57-76 %) together. FP64: the FP64 pipe.
 #pragma once
 
 #include "weo_dslash.cuh"
