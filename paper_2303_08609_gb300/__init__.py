@@ -600,9 +600,8 @@ def wilson_eo_inject_fused_timeout(h, out_e, in_e, stream=None):
 
 def wilson_eo_set_staging(h, staged=True, rows=0, depth=0):
     """Hops of FP32 18-real operators fed by TMA through a shared-memory ring
-    (True or 1: single-RHS hops; 2: multi-RHS hops too) or the default
-    one-site-per-thread kernel (False); rows per tile and ring depth, 0 for
-    automatic."""
+    (True or 1: single-RHS hops; 2: multi-RHS hops too) or the default kernel
+    (False); rows per tile and ring depth, 0 for automatic."""
     _check(_load().wilson_eo_set_staging(h, int(staged), int(rows), int(depth)),
            "wilson_eo_set_staging")
 
