@@ -430,8 +430,8 @@ int wilson_eo_set_rhs_lanes(wilson_eo_t h, int lanes);
  * rows (y0 + dy, z0 + dz, t0 + dt), dy, dz, dt in {0, 1}, so that half of its
  * y, z and t neighbour rows are rows it reads anyway and come from L1 rather
  * than L2 (Sec. 3.2 blocks sites in x and y for the same reason). Used when
- * 64 <= 8 Lx/2 <= 256 (other lattices keep the default kernel); the CTA size then replaces wilson_eo_set_launch's
- * `threads`. The results do not depend on it. WEO_ERR_ARG for other values.
+ * 64 <= 8 Lx/2 <= 256 (other lattices keep the default kernel); the CTA size
+ * then replaces wilson_eo_set_launch's `threads`. The results do not depend on it. WEO_ERR_ARG for other values.
  * wilson_eo_tune times it too. */
 int wilson_eo_set_site_blocks(wilson_eo_t h, int blocked);
 

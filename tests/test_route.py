@@ -80,6 +80,52 @@ MEASURED = """
 32 12 331776 9 523.17 477.03 436.03
 32 12 32768 16 97.32 85.83 91.81
 32 12 131072 6 148.10 128.11 127.69
+16 18 589824 2 183.10 179.44 257.54
+16 18 589824 3 260.89 261.01 311.33
+16 18 589824 4 337.97 343.13 340.26
+16 18 589824 6 489.93 507.57 511.31
+16 18 589824 7 566.02 589.95 569.34
+32 18 589824 2 254.50 232.40 280.25
+32 18 589824 3 354.08 329.01 329.78
+32 18 589824 4 452.50 425.48 369.84
+32 18 589824 6 647.89 621.08 540.04
+32 18 589824 7 748.85 716.73 591.98
+32 12 589824 2 233.71 205.02 269.16
+32 12 589824 3 329.60 295.76 321.27
+32 12 589824 4 426.32 387.66 358.86
+32 12 589824 6 621.12 568.97 532.02
+32 12 589824 7 725.83 660.63 585.54
+16 12 589824 2 176.91 183.81 254.68
+16 12 589824 3 256.87 270.69 308.85
+16 12 589824 4 335.85 357.34 337.59
+16 12 589824 6 495.15 530.73 508.27
+16 12 589824 7 575.28 617.81 566.84
+16 18 1048576 2 315.93 311.52 450.40
+16 18 1048576 3 451.45 454.95 543.68
+16 18 1048576 4 586.97 599.94 588.95
+16 18 1048576 6 860.57 890.66 889.12
+16 18 1048576 7 997.22 1035.94 996.89
+32 18 1048576 2 439.51 409.29 478.49
+32 18 1048576 3 612.72 579.34 563.13
+32 18 1048576 4 781.71 749.34 629.44
+32 18 1048576 6 1140.83 1096.95 940.11
+32 18 1048576 7 1333.53 1276.48 1042.71
+32 12 1048576 2 400.95 360.00 460.55
+32 12 1048576 3 574.80 519.64 551.05
+32 12 1048576 4 756.60 679.85 612.32
+32 12 1048576 6 1114.07 1001.74 922.55
+32 12 1048576 7 1297.27 1170.31 1025.51
+16 12 1048576 2 304.94 322.00 444.69
+16 12 1048576 3 447.00 476.24 539.47
+16 12 1048576 4 587.93 629.98 584.45
+16 12 1048576 6 872.43 937.46 881.55
+16 12 1048576 7 1014.68 1092.77 991.35
+16 18 5308416 2 1563.05 1580.24 2296.16
+16 18 5308416 3 2284.06 2337.27 2797.42
+32 18 5308416 2 2281.02 2099.01 2574.38
+32 12 5308416 3 3065.02 2756.86 3018.95
+16 12 1280000 1 200.21 199.88 9999
+16 12 2048000 1 313.86 316.99 9999
 """
 
 # FP64: link reals, V/2, right-hand sides: rows (16-site CTAs), pairs (32 sites)
