@@ -808,13 +808,14 @@ static int solve_impl(wilson_eo_s *h, double tol, int maxiter, int mixed, int *i
         // the inner system is that of r / scale, |r / scale| in [1, 2) at the start: its
         // residuals' squares stay inside FP32's range whatever that of b is, and a power
         // of two changes no rounding
-        std::vector<double> scale(R, 1.0);
+        std::vector<double> scale(R, 1.0), both(2 * R);  // `both` outlives its copy
         for (int r = 0; r < R; ++r) {
             if (rr_true[r] > 0.0) scale[r] = ldexp(1.0, std::max(-1000, std::min(1000, ilogb(sqrt(rr_true[r])))));
-            const double both[2] = {scale[r], 1.0 / scale[r]};
-            WEO_CUDA(cudaMemcpyAsync(static_cast<char *>(S->scal.ptr) + r * sizeof(SolveScalars) + offsetof(SolveScalars, scale),
-                                     both, sizeof both, cudaMemcpyHostToDevice, s));
+            both[2 * r] = scale[r];
+            both[2 * r + 1] = 1.0 / scale[r];
         }
+        WEO_CUDA(cudaMemcpy2DAsync(static_cast<char *>(S->scal.ptr) + offsetof(SolveScalars, scale), sizeof(SolveScalars),
+                                   both.data(), 2 * sizeof(double), 2 * sizeof(double), R, cudaMemcpyHostToDevice, s));
         WEO_CUDA(cudaMemsetAsync(S->xs.ptr, 0, b32, s));
         k_convert<<<dim3(flat_grid(n), R), 256, 0, s>>>((float2 *)S->rs.ptr, (const double2 *)S->r64.ptr, n, sc);
         WEO_CUDA(cudaMemcpyAsync(S->p.ptr, S->rs.ptr, b32, cudaMemcpyDeviceToDevice, s));

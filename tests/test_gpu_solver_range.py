@@ -25,3 +25,19 @@ def test_solve_of_a_scaled_right_hand_side(prec, fmt, power):
     assert info["converged"] and scaled["converged"], scaled
     assert scaled["iterations"] == info["iterations"]
     assert torch.equal(y, x * 2.0 ** power)
+
+
+@pytest.mark.gpu
+def test_each_right_hand_side_has_its_own_scale():
+    import torch
+
+    import paper_2303_08609_gb300 as weo
+
+    dims = (8, 8, 8, 8)
+    b = to_device(to_planar(gen.gaussian_spinor(dims, nrhs=3, seed=503)))
+    s = torch.tensor([2.0 ** 61, 1.0, 2.0 ** -50], dtype=torch.float64, device="cuda")[:, None, None, None]
+    with weo.WilsonEO(dims, 0.13, to_device(gen.gauge_field(dims, "smooth", seed=501, eps=0.4)), prec="f16") as op:
+        x, info = op.solve(b, tol=1e-10)
+        y, scaled = op.solve(b * s, tol=1e-10)
+    assert info["converged"] and scaled["converged"]
+    assert torch.equal(y, x * s)
